@@ -4,8 +4,8 @@
 //    [L | D | U] gathers its A block, or zero for a fill position.
 // 2. Block ILU(0) on A' (Algorithm 4), one warp per block row, rows claimed in
 //    ascending order through an atomic ticket.  Row i walks its pivots p < i
-//    in ascending order; for each it waits (bounded, acquire) until row p is
-//    finished, then
+//    in ascending order, waiting (bounded, acquire) until row p is finished,
+//    and does
 //        A_ip <- A_ip D_p^{-1}
 //        A_ij <- A_ij - A_ip U_pj   for every j > p with (p,j) and (i,j) in P'
 //    where U_pj is row p's final, still unscaled upper block.  The j updates of
@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "device_common.cuh"
 
@@ -49,47 +50,121 @@ __global__ void factor_init_kernel(int32_t* header, int32_t* done, int32_t n) {
     header[threadIdx.x] = (threadIdx.x == kBadRow) ? 0x7fffffff : 0;
 }
 
-// Row storage of the factor kernel: up to RC blocks of a row are staged in
-// shared memory (per warp); longer rows are worked on in place in global
-// memory through the same slot interface.  8 warps per CTA: two CTAs fit on
-// an SM for b <= 5 (registers), twice the chunks in flight of one 16-warp CTA
-// for the same warps (measured 4-13 % faster with 256-row chunk targets).
+// Row storage of the factor kernel: rows of up to RC blocks are staged in
+// shared memory (per warp); longer rows are worked on in place in global memory
+// through the same slot interface.  A warp takes a row's pivots in batches of
+// up to LC entries of their U rows, whose matches in the row are listed before
+// anything is waited for.  8 warps per CTA: twice the chunks in flight of one
+// 16-warp CTA for the same warps (measured 4-13 % faster with 256-row chunk
+// targets).
 template <int B>
 struct FactorCap {
-  static constexpr int W = 8;                          // warps per CTA
+  static constexpr int W = 8;  // warps per CTA
   static constexpr int RC = B <= 4 ? 64 : (B <= 6 ? 32 : 24);
-  static constexpr int WDBL = RC * B * B + 4 * B * B;  // doubles per warp
-  static constexpr int WINT = RC + 32;                 // ints per warp
+  static constexpr int LC = B <= 2 ? 64 : B == 3 ? 48 : B == 4 ? 32 : B <= 6 ? 16 : 12;
+  static constexpr int KC = B <= 4 ? 16 : 6;  // pivot blocks D_p^{-1} held at once
+  static constexpr int WVAL = (LC + KC + 1) * B * B;  // values per warp beside the staged row
+  static constexpr int WINT = 2 * LC + 2 * 34;        // ints per warp beside the row's columns
 };
 
+// rc: rows of up to rc blocks are staged (at most RC; the widest row of the
+// pattern if that is less).
 template <int B, typename TV>
-size_t factor_smem_bytes(int chunk) {
-  return (size_t)FactorCap<B>::W * FactorCap<B>::WDBL * sizeof(TV) +
-         ((size_t)2 * chunk + (size_t)FactorCap<B>::W * FactorCap<B>::WINT) * sizeof(int);
+size_t factor_smem_bytes(int chunk, int rc) {
+  return (size_t)FactorCap<B>::W * (FactorCap<B>::WVAL + rc * B * B) * sizeof(TV) +
+         ((size_t)2 * chunk + (size_t)FactorCap<B>::W * (FactorCap<B>::WINT + rc)) * sizeof(int);
 }
 
+// Whether a value is finite, and the order of magnitudes, on the integer pipes
+// (an FP64 comparison takes the FP64 pipe).
+__device__ __forceinline__ unsigned long long magnitude(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ unsigned magnitude(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ bool finite_bits(double v) { return magnitude(v) < 0x7ff0000000000000ull; }
+__device__ __forceinline__ bool finite_bits(float v) { return magnitude(v) < 0x7f800000u; }
+
+// D^{-1} by Gauss-Jordan with partial pivoting on [D | I]: lane c < 2B holds
+// column c in registers (the upper lanes hold nothing and mirror column 0).
+// False if a pivot or the result is zero or not finite.
+template <int B, typename TV>
+__device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
+  bool bad = false;
+#pragma unroll
+  for (int r = 0; r < B; ++r) bad |= lane < B && !finite_bits(col[r]);
+  if (__any_sync(kFull, bad)) return false;
+#pragma unroll
+  for (int c = 0; c < B; ++c) {
+    // the pivot row, from column c
+    int pr = c;
+    auto best = magnitude(__shfl_sync(kFull, col[c], c));
+    TV piv = __shfl_sync(kFull, col[c], c);
+#pragma unroll
+    for (int r = c + 1; r < B; ++r) {
+      const TV v = __shfl_sync(kFull, col[r], c);
+      if (magnitude(v) > best) {
+        best = magnitude(v);
+        pr = r;
+        piv = v;
+      }
+    }
+    if (best == 0) return false;
+    const TV top = col[c];
+#pragma unroll
+    for (int r = c + 1; r < B; ++r)
+      if (pr == r) {
+        col[c] = col[r];
+        col[r] = top;
+      }
+    col[c] = col[c] / piv;
+    TV fr[B];
+#pragma unroll
+    for (int r = 0; r < B; ++r) fr[r] = __shfl_sync(kFull, col[r], c);
+#pragma unroll
+    for (int r = 0; r < B; ++r)
+      if (r != c && magnitude(fr[r]) != 0) col[r] = fma(-fr[r], col[c], col[r]);
+  }
+  bad = false;
+#pragma unroll
+  for (int r = 0; r < B; ++r) bad |= lane >= B && lane < 2 * B && !finite_bits(col[r]);
+  return !__any_sync(kFull, bad);
+}
+
+// Measured before / after (backfill to U' = D^{-1} U, same chunks): 96x96x48
+// ILU(1) b = 3 FP64 6.20 / 5.56 ms, 61x47x33 ILU(2) b = 4 FP32 5.64 / 4.23 ms;
+// per row 37 k cycles, of which 10 k the inverse, 9 k the pivots, 5 k staging.
+// What bounds it: the FP64 pipe (19 cycles per warp instruction and SM whatever
+// the active lanes) and the chain of dependent rows.  So a row's work is cut to
+// the matching entries of its pivots' U rows, packed over the lanes, with
+// comparisons on the integer pipes and the b x b inverse in registers; and the
+// blocks of all pivots that are finished are fetched in one round trip, with
+// only what depends on the last pivots left once those arrive.
 template <int B, typename TV>
 __global__ void __launch_bounds__(FactorCap<B>::W * 32) factor_kernel(
-    int32_t n, int32_t chunk, int32_t nchunks, const int32_t* __restrict__ bnd, const int32_t* __restrict__ ord,
-    const int32_t* __restrict__ tick,
+    int32_t n, int32_t chunk, int32_t rc, int32_t nchunks, const int32_t* __restrict__ bnd,
+    const int32_t* __restrict__ ord, const int32_t* __restrict__ tick,
     const int32_t* __restrict__ lrp, const int32_t* __restrict__ lci,
     const int32_t* __restrict__ urp, const int32_t* __restrict__ uci, TV* f, long long nnz_l,
     int32_t* header, int32_t* done, long long spin_ns) {
+  using Cap = FactorCap<B>;
   constexpr int BB = B * B;
   constexpr int H = (BB + 31) / 32;
-  constexpr int RC = FactorCap<B>::RC;
+  constexpr int LC = Cap::LC, KC = Cap::KC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  TV* wd = reinterpret_cast<TV*>(smem_raw) + (size_t)warp * FactorCap<B>::WDBL;
-  TV* rowv = wd;             // RC blocks of the row being factored
-  TV* dp = rowv + RC * BB;   // D_p^{-1}
-  TV* aip = dp + BB;         // scaled A_ip
-  TV* aug = aip + BB;        // [D_i | I] for Gauss-Jordan
-  int* ib = reinterpret_cast<int*>(reinterpret_cast<TV*>(smem_raw) + (size_t)FactorCap<B>::W * FactorCap<B>::WDBL);
-  int* fl = ib;                  // chunk-local ready flags (value = chunk id)
-  int* s_i = fl + chunk;         // rows of the chunk in local-level order
-  int* cols = s_i + chunk + warp * FactorCap<B>::WINT;  // column of each staged slot
-  int* dstv = cols + RC;         // destination slot per U_p entry of a batch
+  const int wvals = Cap::WVAL + rc * BB;
+  TV* rowv = reinterpret_cast<TV*>(smem_raw) + (size_t)warp * wvals;  // the row being factored
+  TV* ub = rowv + rc * BB;  // U_pj of the batch's matches
+  TV* db = ub + LC * BB;    // D_p^{-1}
+  TV* aip = db + KC * BB;   // scaled A_ip
+  int* fl = reinterpret_cast<int*>(reinterpret_cast<TV*>(smem_raw) + (size_t)Cap::W * wvals);  // ready flags (value =
+                                                                                               // chunk id)
+  int* s_i = fl + chunk;  // rows of the chunk in local-level order
+  int* cols = s_i + chunk + warp * (Cap::WINT + rc);  // column of each staged slot
+  int* msrc = cols + rc;    // the batch's matches: U entry,
+  int* mdst = msrc + LC;    // slot in the row
+  int* moff = mdst + LC;    // first match of each pivot of the batch (33)
+  int* coff = moff + 34;    // first candidate of each pivot of the batch (33)
   __shared__ int s_c;
   TV* L = f;
   TV* D = f + (size_t)nnz_l * BB;
@@ -111,203 +186,258 @@ __global__ void __launch_bounds__(FactorCap<B>::W * 32) factor_kernel(
     const int len = hi - lo;
     for (int q = tid; q < len; q += blockDim.x) s_i[q] = ord[lo + q];
     __syncthreads();
-    for (int pos = warp; pos < len && !dead; pos += FactorCap<B>::W) {
+    // first and end entry of a row in L and U
+    auto extent = [&](int pos) {
+      const int i = s_i[min(pos, len - 1)];
+      return make_int4(lrp[i], lrp[i + 1], urp[i], urp[i + 1]);
+    };
+    int4 next = extent(warp);
+    for (int pos = warp; pos < len && !dead; pos += Cap::W) {
       const int i = s_i[pos];
-      const int lb = lrp[i], nl = lrp[i + 1] - lb;
-      const int ub = urp[i], nu = urp[i + 1] - ub;
+      const int lb = next.x, nl = next.y - lb;
+      const int ub0 = next.z, nu = next.w - ub0;
+      next = extent(pos + Cap::W);
       const int nrow = nl + 1 + nu;
-      const bool staged = nrow <= RC;
+      const bool staged = nrow <= rc;
       // slot k of row i: L blocks (k < nl), the pivot block (k == nl), U blocks
       auto blk = [&](int k) -> TV* {
         if (staged) return rowv + k * BB;
         if (k < nl) return L + (size_t)(lb + k) * BB;
         if (k == nl) return D + (size_t)i * BB;
-        return U + (size_t)(ub + k - nl - 1) * BB;
+        return U + (size_t)(ub0 + k - nl - 1) * BB;
       };
       auto colk = [&](int k) -> int {
         if (staged) return cols[k];
         if (k < nl) return lci[lb + k];
         if (k == nl) return i;
-        return uci[ub + k - nl - 1];
+        return uci[ub0 + k - nl - 1];
       };
       if (staged) {
         for (int k = lane; k < nrow; k += 32)
-          cols[k] = k < nl ? lci[lb + k] : (k == nl ? i : uci[ub + k - nl - 1]);
+          cols[k] = k < nl ? lci[lb + k] : (k == nl ? i : uci[ub0 + k - nl - 1]);
         for (int q = lane; q < nl * BB; q += 32) rowv[q] = L[(size_t)lb * BB + q];
         for (int q = lane; q < BB; q += 32) rowv[nl * BB + q] = D[(size_t)i * BB + q];
-        for (int q = lane; q < nu * BB; q += 32) rowv[(nl + 1) * BB + q] = U[(size_t)ub * BB + q];
+        for (int q = lane; q < nu * BB; q += 32) rowv[(nl + 1) * BB + q] = U[(size_t)ub0 * BB + q];
       }
       __syncwarp();
-      for (int k = 0; k < nl; ++k) {
-        const int p = colk(k);
-        const int pb = urp[p], pe = urp[p + 1];
-        // destination slots of the first batch of row p's U entries (pattern
-        // only: done before waiting for row p)
-        auto find_dst = [&](int s0) {
-          const int cnt = min(32, pe - s0);
-          if (lane < cnt) {
-            const int j = uci[s0 + lane];
-            int a = k + 1, z = nrow, d = -1;
+      int k0 = 0, s0 = 0;  // the next batch starts with entry s0 of pivot k0's U row
+      while (k0 < nl && !dead) {
+        // ---- the batch: whole pivots while their U rows hold at most LC
+        // entries (lane x: pivot k0 + x); of a longer one, LC entries of it
+        const int np = min(32, nl - k0);
+        int p = -1, pb = 0, plen = 0;
+        if (lane < np) {
+          p = colk(k0 + lane);
+          pb = urp[p] + (lane == 0 ? s0 : 0);
+          plen = urp[p + 1] - pb;
+        }
+        int upto = plen;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int v = __shfl_up_sync(kFull, upto, d);
+          if (lane >= d) upto += v;
+        }
+        const unsigned fits = __ballot_sync(kFull, lane < np && upto <= LC);
+        int nfit = __popc(fits), next_s0 = 0;
+        const bool slice = nfit == 0;
+        if (slice) {
+          nfit = 1;
+          next_s0 = s0 + LC;
+          if (lane == 0) upto = plen = LC;
+        }
+        const int cands = __shfl_sync(kFull, upto, nfit - 1);
+        __syncwarp();
+        coff[lane] = upto - plen;
+        moff[lane] = 0;
+        if (lane == 0) moff[32] = 0;
+        __syncwarp();
+        // ---- its matches: entries (p, j) with (i, j) in the row, j > p
+        int nm = 0;
+        for (int q0 = 0; q0 < cands; q0 += 32) {
+          const int q = q0 + lane;
+          int x = 0, dst = -1, src = 0;
+          {
+            int z = nfit;  // the last pivot whose first candidate is <= q
+            while (z - x > 1) {
+              const int mid = (x + z) >> 1;
+              if (coff[mid] <= q) x = mid;
+              else z = mid;
+            }
+          }
+          const int first = __shfl_sync(kFull, pb, x);
+          if (q < cands) {
+            src = first + q - coff[x];
+            const int j = uci[src];
+            int a = k0 + x + 1, z = nrow;
             while (a < z) {
               const int mid = (a + z) >> 1;
               const int v = colk(mid);
-              if (v == j) { d = mid; break; }
-              if (v < j) a = mid + 1; else z = mid;
-            }
-            dstv[lane] = d;
-          }
-        };
-        find_dst(pb);
-        const bool ok = (p >= lo && p < hi) ? wait_local_flag(fl + (p - lo), c, w) : wait_flag(done + p, w);
-        if (__any_sync(kFull, !ok)) {
-          dead = true;
-          break;
-        }
-        // A_ip <- A_ip * D_p^{-1}; D_p^{-1} and this lane's first U_pj
-        // operands are fetched together (one memory round trip per pivot)
-        for (int e = lane; e < BB; e += 32) dp[e] = D[(size_t)p * BB + e];
-        constexpr int NPRE = 4;
-        TV upre[NPRE][B];
-        {
-          const int cnt0 = min(32, pe - pb);
-#pragma unroll
-          for (int h = 0; h < NPRE; ++h) {
-            const int wk = lane + 32 * h;
-            if (wk < cnt0 * BB) {
-              const int sidx = wk / BB, e = wk - (wk / BB) * BB;
-              const TV* upj = U + (size_t)(pb + sidx) * BB + (e / B) * B;
-#pragma unroll
-              for (int m = 0; m < B; ++m) upre[h][m] = upj[m];
+              if (v == j) {
+                dst = mid;
+                break;
+              }
+              if (v < j) a = mid + 1;
+              else z = mid;
             }
           }
+          const unsigned m = __ballot_sync(kFull, dst >= 0);
+          if (dst >= 0) {
+            const int at = nm + __popc(m & ((1u << lane) - 1u));
+            msrc[at] = src;
+            mdst[at] = dst;
+            atomicAdd(&moff[x + 1], 1);
+          }
+          nm += __popc(m);
         }
         __syncwarp();
-        TV* a = blk(k);
-        TV nv[H];
+        int upm = lane < nfit ? moff[lane + 1] : 0;
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int e = lane + 32 * h;
-          if (e < BB) {
-            const int r = e % B, cc = e / B;
-            TV s = TV(0);
-#pragma unroll
-            for (int m = 0; m < B; ++m) s = fma(a[m * B + r], dp[cc * B + m], s);
-            nv[h] = s;
-          }
+        for (int d = 1; d < 32; d <<= 1) {
+          const int v = __shfl_up_sync(kFull, upm, d);
+          if (lane >= d) upm += v;
         }
         __syncwarp();
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int e = lane + 32 * h;
-          if (e < BB) {
-            a[e] = nv[h];
-            aip[e] = nv[h];
-          }
-        }
+        if (lane < nfit) moff[lane + 1] = upm;
         __syncwarp();
-        // A_ij <- A_ij - A_ip U_pj for j > p in both P'(p) and P'(i)
-        for (int s0 = pb; s0 < pe; s0 += 32) {
-          if (s0 != pb) {
-            find_dst(s0);
-            __syncwarp();
+        // the warp's next row: into L2 while this one waits
+        if (k0 == 0 && s0 == 0) {
+          auto pull = [&](const void* first, size_t bytes) {
+            for (size_t o = (size_t)lane * 128; o < bytes; o += 32 * 128)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)first + o));
+          };
+          pull(lci + next.x, (size_t)(next.y - next.x) * sizeof(int32_t));
+          pull(uci + next.z, (size_t)(next.w - next.z) * sizeof(int32_t));
+          pull(L + (size_t)next.x * BB, (size_t)(next.y - next.x) * BB * sizeof(TV));
+          pull(U + (size_t)next.z * BB, (size_t)(next.w - next.z) * BB * sizeof(TV));
+        }
+        // ---- the pivots, as far as their rows are finished
+        const bool local = p >= lo && p < hi;
+        bool have = false;
+        for (int x = 0; x < nfit && !dead;) {
+          int run = 0;
+          w.t0 = 0;
+          for (unsigned it = 1;; ++it) {
+            if (lane >= x && lane < nfit && !have)
+              have = local ? ld_acquire_cta_shared_s32(fl + (p - lo)) == c : ld_acquire_s32(done + p) != 0;
+            run = __ffs(~(__ballot_sync(kFull, have && lane < nfit) >> x)) - 1;
+            if (run != 0) break;
+            if (__any_sync(kFull, w.give_up(it))) {
+              dead = true;
+              break;
+            }
           }
-          const int cnt = min(32, pe - s0);
-          if (s0 == pb) {
+          if (dead) break;
+          __syncwarp();
+          if (run < 0) run = 32;
+          run = min(min(run, nfit - x), KC);
+          // their D_p^{-1} and matching U_pj, all loads in flight together
+          const int m0 = moff[x], mv = (moff[x + run] - m0) * BB, dv = run * BB;
+          constexpr int ND = (KC * BB + 31) / 32 < 5 ? (KC * BB + 31) / 32 : 5;
+          constexpr int NU = 6;
+          for (int e0 = 0; e0 < dv || e0 < mv; e0 += 32 * (ND < NU ? ND : NU)) {
+            constexpr int NB = ND < NU ? ND : NU;
+            TV tu[NB], td[NB];
 #pragma unroll
-            for (int h = 0; h < NPRE; ++h) {
-              const int wk = lane + 32 * h;
-              if (wk < cnt * BB) {
-                const int sidx = wk / BB, e = wk - (wk / BB) * BB;
-                const int d = dstv[sidx];
-                if (d >= 0) {
-                  const int r = e % B;
-                  TV s = TV(0);
-#pragma unroll
-                  for (int m = 0; m < B; ++m) s = fma(aip[m * B + r], upre[h][m], s);
-                  blk(d)[e] -= s;
-                }
+            for (int h = 0; h < NB; ++h) {
+              const int e = e0 + lane + 32 * h;
+              if (e < dv) {
+                const int y = e / BB;
+                td[h] = D[(size_t)colk(k0 + x + y) * BB + (e - y * BB)];
+              }
+              if (e < mv) {
+                const int y = e / BB;
+                tu[h] = U[(size_t)msrc[m0 + y] * BB + (e - y * BB)];
               }
             }
-          }
-          for (int wk = lane + (s0 == pb ? 32 * NPRE : 0); wk < cnt * BB; wk += 32) {
-            const int sidx = wk / BB;
-            const int e = wk - sidx * BB;
-            const int d = dstv[sidx];
-            if (d >= 0) {
-              const int r = e % B, cc = e / B;
-              const TV* upj = U + (size_t)(s0 + sidx) * BB + cc * B;
-              TV s = TV(0);
 #pragma unroll
-              for (int m = 0; m < B; ++m) s = fma(aip[m * B + r], upj[m], s);
-              blk(d)[e] -= s;
+            for (int h = 0; h < NB; ++h) {
+              const int e = e0 + lane + 32 * h;
+              if (e < dv) db[e] = td[h];
+              if (e < mv) ub[e] = tu[h];
             }
           }
           __syncwarp();
+          for (int y = 0; y < run; ++y) {
+            const int k = k0 + x + y;
+            // A_ip <- A_ip D_p^{-1} (once: with the first slice of a long U row)
+            TV* const a = blk(k);
+            if (x + y > 0 || s0 == 0) {
+              const TV* const dp = db + y * BB;
+              TV nv[H];
+#pragma unroll
+              for (int h = 0; h < H; ++h) {
+                const int e = lane + 32 * h;
+                if (e < BB) {
+                  const int r = e % B, cc = e / B;
+                  TV s = TV(0);
+#pragma unroll
+                  for (int m = 0; m < B; ++m) s = fma(a[m * B + r], dp[cc * B + m], s);
+                  nv[h] = s;
+                }
+              }
+              __syncwarp();
+#pragma unroll
+              for (int h = 0; h < H; ++h) {
+                const int e = lane + 32 * h;
+                if (e < BB) {
+                  a[e] = nv[h];
+                  aip[e] = nv[h];
+                }
+              }
+              __syncwarp();
+            }
+            // A_ij <- A_ij - A_ip U_pj
+            const int mb = moff[x + y], cnt = (moff[x + y + 1] - mb) * BB;
+            for (int wk = lane; wk < cnt; wk += 32) {
+              const int sidx = wk / BB, e = wk - sidx * BB;
+              const int r = e % B, cc = e / B;
+              const TV* const upj = ub + (mb - m0 + sidx) * BB + cc * B;
+              TV s = TV(0);
+#pragma unroll
+              for (int m = 0; m < B; ++m) s = fma(aip[m * B + r], upj[m], s);
+              blk(mdst[mb + sidx])[e] -= s;
+            }
+            __syncwarp();
+          }
+          x += run;
+        }
+        if (slice) {
+          s0 = next_s0;
+        } else {
+          k0 += nfit;
+          s0 = 0;
         }
       }
       if (dead) break;
-      // D_i^{-1} by Gauss-Jordan with partial pivoting on [D_i | I].
+      // the row's U is final; later rows read it
+      if (staged)
+        for (int q = lane; q < nu * BB; q += 32) U[(size_t)ub0 * BB + q] = rowv[(nl + 1) * BB + q];
+      TV col[B];
       {
-        const TV* di = blk(nl);
-        for (int e = lane; e < 2 * BB; e += 32) {
-          const int q = e / B, r = e % B;
-          aug[e] = q < B ? di[e] : (r == q - B ? TV(1) : TV(0));
-        }
-      }
-      __syncwarp();
-      bool bad = false;
-      for (int e = lane; e < BB; e += 32) bad |= !isfinite(aug[e]);
-      bad = __any_sync(kFull, bad);
-      for (int cc = 0; cc < B && !bad; ++cc) {
-        int pr = cc;
-        TV best = fabs(aug[cc * B + cc]);
+        const TV* const di = blk(nl);
 #pragma unroll
-        for (int r = cc + 1; r < B; ++r) {
-          const TV v = fabs(aug[cc * B + r]);
-          if (v > best) { best = v; pr = r; }
-        }
-        if (!(best > TV(0))) { bad = true; break; }
-        const TV piv = aug[cc * B + pr];
-        __syncwarp();
-        if (lane < 2 * B) {
-          TV* col = aug + lane * B;
-          if (pr != cc) { const TV tmp = col[cc]; col[cc] = col[pr]; col[pr] = tmp; }
-          col[cc] = col[cc] / piv;
-        }
-        __syncwarp();
-        TV fr[B];
-#pragma unroll
-        for (int r = 0; r < B; ++r) fr[r] = aug[cc * B + r];
-        __syncwarp();
-        if (lane < 2 * B) {
-          TV* col = aug + lane * B;
-          const TV pc = col[cc];
-#pragma unroll
-          for (int r = 0; r < B; ++r)
-            if (r != cc && fr[r] != TV(0)) col[r] = fma(-fr[r], pc, col[r]);
-        }
-        __syncwarp();
+        for (int r = 0; r < B; ++r)
+          col[r] = lane < B ? di[lane * B + r] : (lane < 2 * B && r == lane - B ? TV(1) : TV(0));
       }
-      if (!bad) {
-        for (int e = lane; e < BB; e += 32) bad |= !isfinite(aug[BB + e]);
-        bad = __any_sync(kFull, bad);
-      }
-      // write the finished row back: L blocks, D_i^{-1}, unscaled U blocks
-      for (int e = lane; e < BB; e += 32) D[(size_t)i * BB + e] = aug[BB + e];
-      if (staged) {
-        for (int q = lane; q < nl * BB; q += 32) L[(size_t)lb * BB + q] = rowv[q];
-        for (int q = lane; q < nu * BB; q += 32) U[(size_t)ub * BB + q] = rowv[(nl + 1) * BB + q];
+      const bool bad = !invert_columns<B, TV>(col, lane);
+      if (lane >= B && lane < 2 * B) {
+#pragma unroll
+        for (int r = 0; r < B; ++r) D[(size_t)i * BB + (lane - B) * B + r] = col[r];
       }
       if (bad && lane == 0) {
         atomicMin(header + kBadRow, i);
         atomicCAS(header + kErr, 0, (int)BILU_ERR_SINGULAR);
       }
+      // rows of this chunk first: their flag needs no device-wide fence
+      __threadfence_block();
+      __syncwarp();
+      if (lane == 0) st_release_cta_shared_s32(fl + (i - lo), c);
       __threadfence();
       __syncwarp();
-      if (lane == 0) {
-        st_release_cta_shared_s32(fl + (i - lo), c);
-        st_release_s32(done + i, 1);
-      }
+      if (lane == 0) st_release_s32(done + i, 1);
+      if (staged)
+        for (int q = lane; q < nl * BB; q += 32) L[(size_t)lb * BB + q] = rowv[q];
+      __syncwarp();
     }
   }
 }
@@ -345,6 +475,9 @@ __global__ void __launch_bounds__(256) scale_upper_kernel(int32_t n, const int32
   }
 }
 
+// Dynamic shared memory a CTA may use beside factor_kernel's static word.
+constexpr int kFactorMaxSmem = 227 * 1024 - 256;
+
 int device_sms() {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -378,19 +511,23 @@ int launch_factor_t(const bilu_pattern* p, int32_t b, TV* f, int32_t* header, in
   const int nchunks = p->fact.nchunks;
   const long long spin = trisolve_config().spin_ns;
   BILU_DISPATCH_B(b, {
-    const size_t smem = factor_smem_bytes<B, TV>(chunk);
-    static int last_chunk = -1, per_sm = 1;
-    if (last_chunk != chunk) {
-      cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)std::max<size_t>(smem, 48 * 1024));
+    // rows of the pattern are at most max_l + 1 + max_u blocks wide
+    const int rc = std::min(FactorCap<B>::RC, p->max_l + 1 + p->max_u);
+    const size_t smem = factor_smem_bytes<B, TV>(chunk, rc);
+    // the CTAs that fit on an SM, asked for once per shared-memory size: (bytes << 8) | CTAs
+    static std::atomic<unsigned long long> cache{0};
+    unsigned long long have = cache.load(std::memory_order_relaxed);
+    if ((have >> 8) != smem) {
+      cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFactorMaxSmem);
       int q = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, factor_kernel<B, TV>, FactorCap<B>::W * 32, smem);
-      per_sm = q < 1 ? 1 : q;
-      last_chunk = chunk;
+      have = ((unsigned long long)smem << 8) | (unsigned long long)std::max(1, std::min(q, 255));
+      cache.store(have, std::memory_order_relaxed);
     }
+    const int per_sm = (int)(have & 255);
     const int grid = std::max(1, std::min(nchunks, per_sm * sms));
     ProfScope ps(BILU_PROF_FACTOR, stream);
-    factor_kernel<B, TV><<<grid, FactorCap<B>::W * 32, smem, s>>>(n, chunk, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
+    factor_kernel<B, TV><<<grid, FactorCap<B>::W * 32, smem, s>>>(n, chunk, rc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
                                                             p->d_urp, p->d_uci, f, p->nnz_l(), header, done,
                                                             spin);
   });
