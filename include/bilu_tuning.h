@@ -35,9 +35,11 @@ int32_t bilu_get_trisolve_chunk(void);
 int32_t bilu_auto_trisolve_chunk(const bilu_pattern* p);
 
 /* Target of consecutive block rows one CTA owns in the sync-free
- * factorization: 0 (the default) picks n / (2 * SMs) clamped to [64, 256],
- * or 3 L (three grid lines) where that hits 256 and a line length L of
- * 16..128 rows is detected (see bilu_set_trisolve_chunk);
+ * factorization: 0 (the default) picks whole grid lines where a line length L
+ * of 16..128 rows is detected (see bilu_set_trisolve_chunk) -- L where the
+ * widest row of L or U' has more than 8 blocks, 2 L where it has more than 4
+ * and n / (2 * SMs) < 1024, else 3 L (2 L where n / (2 * SMs) < 256) -- and
+ * n / (2 * SMs) clamped to [64, 256] without one;
  * 1 <= rows <= 1024 fixes it; other values: BILU_ERR_ARG.  Its schedule is
  * separate from the solves'; like theirs it is built by bilu_pattern_upload
  * and bilu_pattern_schedule only. */

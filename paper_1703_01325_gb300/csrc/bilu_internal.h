@@ -116,8 +116,9 @@ TrisolveConfig& trisolve_config();
 // The chunk targets in effect for a pattern of n block rows: the configured
 // ones, or (0) n / (10 * SMs) in [32, 256] for the solves and n / (2 * SMs)
 // in [64, 256] for the factorization -- enough chunks to fill the GPU --
-// except on large grids with a detected line length L: 2 L for the solves
-// (16 <= L <= 192), 3 L for the factorization (16 <= L <= 128).
+// except with a detected line length L: 2 L for the solves of large grids
+// (16 <= L <= 192), L to 3 L by row width for the factorization (16 <= L <=
+// 128).
 int32_t solve_chunk_target(const bilu_pattern* p);
 int32_t auto_solve_chunk_target(const bilu_pattern* p);  // the rule alone
 int32_t factor_chunk_target(const bilu_pattern* p);

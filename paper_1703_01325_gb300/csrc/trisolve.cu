@@ -91,11 +91,22 @@ int32_t solve_chunk_target(const bilu_pattern* p) {
   return c > 0 ? c : auto_solve_chunk_target(p);
 }
 
-// The factorization's 8-warp CTAs do best with three grid lines per chunk on
-// large grids (128-wide: 12.4 ms against 13.7 with two lines).
+// The factorization's 8-warp CTAs: whole grid lines, the fewer the wider the
+// rows.  A warp's row takes time in its number of pivots, and a chunk of more
+// lines gives each level more rows than its warps finish in the time a level
+// of narrow rows takes; fewer lines hold fewer rows in flight.  Measured with
+// 1 / 2 / 3 lines (ms, FP64): 96x96x48 7-point b = 3, widest row of 6 blocks:
+// 8.6 / 5.7 / 5.6; 64x64x32 the same rows: 3.0 / 2.3 / 2.7; 61x47x33 b = 5, 3
+// blocks: 3.6 / 2.5 / 2.3; 61x47x33 b = 4, 11 blocks: 4.7 / 6.3 / 8.2; 27-point
+// 40x40x20 b = 3, 25 blocks: 6.4 / 10.2 / 17.5 (62 with 105 rows, which cut
+// lines), 80x80x40 ILU(2): 117 / 182 / 292.
 int32_t auto_factor_chunk_target(const bilu_pattern* p) {
   const long long t = (long long)p->n / (2LL * device_sm_count());
-  if (t >= 256 && p->line_len >= 16 && p->line_len <= 128) return 3 * p->line_len;
+  if (p->line_len >= 16 && p->line_len <= 128) {
+    const int widest = std::max(p->max_l, p->max_u);
+    const int lines = widest > 8 ? 1 : widest > 4 && t < 1024 ? 2 : t >= 256 ? 3 : 2;
+    return lines * p->line_len;
+  }
   return (int32_t)std::max(64LL, std::min(256LL, t));
 }
 
