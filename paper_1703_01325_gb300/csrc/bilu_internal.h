@@ -186,7 +186,6 @@ void ticket_order_lists(int32_t nchunks, const std::vector<int32_t>& prio, const
 int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
 // Eq. 4 levels, L / U' split and backfill map of a pattern with rp, ci, lev set.
 int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col_idx);
-int validate_pattern(int32_t n, const int32_t* row_ptr, const int32_t* col_idx);
 // Fills the host vectors of a device-built pattern from its device copies
 // (cudaMemcpy only; the current device must hold them).  Set-up/host calls.
 int ensure_host(const bilu_pattern* p);

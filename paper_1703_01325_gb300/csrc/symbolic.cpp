@@ -148,12 +148,6 @@ int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col
   return BILU_OK;
 }
 
-// The block CSR checks of bilu_symbolic (sorted, unique, in range, diagonal
-// present), for the device symbolic phase.
-int validate_pattern(int32_t n, const int32_t* row_ptr, const int32_t* col_idx) {
-  return check_pattern(n, row_ptr, col_idx);
-}
-
 }  // namespace bilu
 
 extern "C" int bilu_symbolic(int32_t n, const int32_t* row_ptr, const int32_t* col_idx, int32_t k,

@@ -1,7 +1,17 @@
 // symbolic_gpu.cu -- the symbolic phase (Section 2.2, Algorithm 3 with Eq. 1
 // and Eq. 2) on the device, bit-identical to the host phase in symbolic.cpp.
 //
-// Row i of P' is the same pivot-driven merge as on the host: start from A's
+// Two ways to the same P' and levels:
+//
+// By paths (path_kernel; k <= kMaxPathLevel).  The level of fill of (i, j) is
+// one less than the length of the shortest path from i to j in A's graph whose
+// interior vertices are all numbered below min(i, j) (the fill-path theorem of
+// Rose and Tarjan, for levels Hysom and Pothen).  So every row can be found from
+// A alone, without any other row of P': no row waits, where the merge below is a
+// chain over the rows' dependency levels.  One warp per row.
+//
+// By merges (symbolic_kernel), for larger k and rows the path kernel's tables do
+// not hold.  Row i of P' is the same pivot-driven merge as on the host: start from A's
 // row (Eq. 1: level 0), take the pivots p < i of level <= k in ascending
 // column order (a pivot's level is final when it is reached, since only
 // smaller pivots lower it), and for each merge row p's final upper part into
@@ -190,11 +200,224 @@ __global__ void __launch_bounds__(kSymWarps * 32) symbolic_kernel(
   }
 }
 
+// ---- rows of P' by paths ----
+
+// Statistics words (device scratch).
+enum StatWord : int { kMaxL = 0, kMaxU = 1, kNlevL = 2, kNlevU = 3, kBadPattern = 4, kLongest = 5, kStatWords = 8 };
+
+constexpr int kMaxPathLevel = 3;  // longer walks revisit more than a merge does
+constexpr int kPathWarps = 4;
+constexpr int kNever = INT_MAX;
+
+// The checks of bilu_symbolic on the device: row pointers ascending and within
+// nnz before a row's columns are looked at, columns sorted, unique, in range,
+// the diagonal present.
+__global__ void check_kernel(int32_t n, int32_t nnz, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                             int32_t* bad, int32_t* longest) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  int lng = 0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const int beg = rp[i], end = rp[i + 1];
+    bool ok = beg >= 0 && beg <= end && end <= nnz;
+    if (ok) {
+      bool diag = false;
+      int prev = -1;
+      for (int t = beg; t < end && ok; ++t) {
+        const int j = ci[t];
+        ok = j > prev && j < n;
+        diag |= j == (int)i;
+        prev = j;
+      }
+      ok = ok && diag;
+      lng = max(lng, end - beg);
+    }
+    if (!ok) *bad = 1;
+  }
+  lng = __reduce_max_sync(kFull, lng);
+  if ((threadIdx.x & 31) == 0) atomicMax(longest, lng);
+}
+
+// Shared memory of a warp of the path kernel, in ints: a hash table of the
+// vertices met (HS slots: column, level, the least possible largest interior
+// vertex of a walk of the current and of the next length, A's entry), the slots
+// in use, and the accepted entries.
+template <int HS>
+struct PathTable {
+  static constexpr int kMost = HS * 3 / 4;  // vertices held
+  static constexpr int kInts = 5 * HS + 3 * kMost + 4;
+};
+
+// Row i by walks of length 1 .. k + 1 from i.  Of the walks of one length that
+// end in v, the one whose largest interior vertex is least decides: it is a fill
+// path iff that vertex is below min(i, v), and only it need be continued (interior
+// vertices are below i).  GL lanes share the neighbours of one vertex.
+//   emit = false: counts only (len, nl, nu, flag as in row_info_kernel);
+//   emit = true: the row itself, and its slots' blocks of A.
+// A row that does not fit the table or has more than `cap` entries sets
+// header[kErr] (the caller turns to a larger table or to the merges).
+template <int HS, int GL>
+__global__ void __launch_bounds__(kPathWarps * 32) path_kernel(
+    int32_t n, int32_t k, int32_t cap, bool emit, const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
+    int32_t* __restrict__ olen, int32_t* __restrict__ nl, int32_t* __restrict__ nu, int32_t* __restrict__ flag,
+    int32_t* stats, const int32_t* __restrict__ rp, const int32_t* __restrict__ lrp, const int32_t* __restrict__ urp,
+    long long nnz_l, int32_t* __restrict__ ci, int32_t* __restrict__ lev, int32_t* __restrict__ lci,
+    int32_t* __restrict__ uci, int32_t* __restrict__ slot_src, int32_t* header) {
+  using T = PathTable<HS>;
+  extern __shared__ int path_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int* const key = path_smem + warp * T::kInts;
+  int* const best = key + HS;   // smallest level found
+  int* const src = best + HS;   // A's entry
+  int* cur = src + HS;          // walks of the current length: least largest interior vertex
+  int* next = cur + HS;
+  int* const used = next + HS;  // slots in use
+  int* const acol = used + T::kMost;
+  int* const aslot = acol + T::kMost;
+  int* const count = aslot + T::kMost;
+  const long long nw = (long long)gridDim.x * kPathWarps;
+  int most_l = 0, most_u = 0;
+  for (long long row = (long long)blockIdx.x * kPathWarps + warp; row < n; row += nw) {
+    const int i = (int)row;
+    for (int q = lane; q < HS; q += 32) {
+      key[q] = -1;
+      best[q] = kNever;
+      src[q] = -1;
+      cur[q] = kNever;
+      next[q] = kNever;
+    }
+    if (lane == 0) *count = 0;
+    __syncwarp();
+    // The slot of column v, a new one if need be; -1: the table is full.
+    auto slot_of = [&](int v) {
+      unsigned h = ((unsigned)v * 2654435761u >> 16) & (HS - 1);
+      for (int tries = 0; tries < HS; ++tries) {
+        const int was = atomicCAS(key + h, -1, v);
+        if (was == v) return (int)h;
+        if (was == -1) {
+          const int at = atomicAdd(count, 1);
+          if (at >= T::kMost) return -1;
+          used[at] = (int)h;
+          return (int)h;
+        }
+        h = (h + 1) & (HS - 1);
+      }
+      return -1;
+    };
+    bool full = false;
+    const int ab = arp[i], ae = arp[i + 1];
+    for (int t = ab + lane; t < ae; t += 32) {  // Eq. 1
+      const int s = slot_of(aci[t]);
+      if (s < 0) {
+        full = true;
+        break;
+      }
+      best[s] = 0;
+      src[s] = t;
+      cur[s] = -1;  // no interior vertex
+    }
+    full = __any_sync(kFull, full);
+    __syncwarp();
+    for (int d = 1; d <= k && !full; ++d) {  // walks of length d + 1
+      const int len = min(*count, T::kMost);
+      __syncwarp();
+      for (int q0 = 0; q0 < len && !full; q0 += 32 / GL) {
+        const int q = q0 + lane / GL;
+        int u = i, top = kNever;
+        if (q < len) {
+          const int s = used[q];
+          u = key[s];
+          top = cur[s];
+        }
+        if (u < i && top != kNever) {
+          top = max(top, u);
+          const int ue = arp[u + 1];
+          for (int t = arp[u] + lane % GL; t < ue; t += GL) {
+            const int v = aci[t];
+            const bool path = top < min(i, v);
+            // of the longest walks, only those that are fill paths count
+            if (v == i || v == u || (d == k && !path)) continue;
+            const int s = slot_of(v);
+            if (s < 0) {
+              full = true;
+              break;
+            }
+            if (path) atomicMin(best + s, d);
+            if (v < i) atomicMin(next + s, top);
+          }
+        }
+        full = __any_sync(kFull, full);
+      }
+      __syncwarp();
+      int* const t = cur;
+      cur = next;
+      next = t;
+      for (int q = lane; q < HS; q += 32) next[q] = kNever;
+      __syncwarp();
+    }
+    // the entries of the row: the vertices some fill path reaches
+    const int len = min(*count, T::kMost);
+    int m = 0, lower = 0;
+    bool after = false;  // whether the row depends on its predecessor
+    for (int q0 = 0; q0 < len; q0 += 32) {
+      const int s = q0 + lane < len ? used[q0 + lane] : 0;
+      const int v = key[s];
+      const bool in = q0 + lane < len && best[s] <= k;
+      const unsigned mask = __ballot_sync(kFull, in);
+      if (in) {
+        const int at = m + __popc(mask & ((1u << lane) - 1u));
+        acol[at] = v;
+        aslot[at] = s;
+      }
+      lower += __popc(__ballot_sync(kFull, in && v < i));
+      after = after || __any_sync(kFull, in && v == i - 1);
+      m += __popc(mask);
+    }
+    __syncwarp();
+    if (full || m > cap) {
+      if (lane == 0) atomicCAS(header + kErr, 0, (int)BILU_ERR_OOM);
+      continue;
+    }
+    if (!emit) {
+      if (lane == 0) {
+        olen[i] = m;
+        nl[i] = lower;
+        nu[i] = m - lower - 1;
+        flag[i] = after ? 0 : 1;
+      }
+      most_l = max(most_l, lower);
+      most_u = max(most_u, m - lower - 1);
+      continue;
+    }
+    const int pb = rp[i], lb = lrp[i], ub = urp[i];
+    for (int q = lane; q < m; q += 32) {
+      const int v = acol[q], s = aslot[q];
+      int rank = 0;  // columns before v
+      for (int x = 0; x < m; ++x) rank += acol[x] < v;
+      ci[pb + rank] = v;
+      lev[pb + rank] = best[s];
+      long long slot;
+      if (v < i) {
+        lci[lb + rank] = v;
+        slot = lb + rank;
+      } else if (v == i) {
+        slot = nnz_l + i;
+      } else {
+        uci[ub + rank - lower - 1] = v;
+        slot = nnz_l + n + ub + (rank - lower - 1);
+      }
+      slot_src[slot] = src[s];
+    }
+    __syncwarp();
+  }
+  if (!emit && lane == 0) {
+    atomicMax(stats + kMaxL, most_l);
+    atomicMax(stats + kMaxU, most_u);
+  }
+}
+
 // ---- completion of the pattern on the device (Eq. 4, L / U' split,
 // backfill map), so that no host pass over P' is needed ----
 
-// Statistics words (device scratch).
-enum StatWord : int { kMaxL = 0, kMaxU = 1, kNlevL = 2, kNlevU = 3, kStatWords = 8 };
 
 // Per row of P' (capacity layout, columns sorted, the diagonal present): its
 // length, the blocks left (nl) and right (nu) of the diagonal, and whether
@@ -321,56 +544,75 @@ __device__ __forceinline__ void st_relaxed_s32(int32_t* p, int v) {
 // Eq. 4 on the device: l(i) = 1 + max l(j) over the dependencies j of row i
 // (0 for a row without any), 0-based, for L (j < i, rows ascending) or for
 // the reversed graph of U' (j > i, rows descending).  Sync-free: warps claim
-// rows in solve order through a ticket, so a row only waits on rows whose
-// tickets were handed out before, all held by running warps; done[j] holds
-// l(j) + 1 once known (0 = pending) and is itself the flag.  The waits are
-// warp-uniform (the whole warp re-reads until no lane sees a pending value)
-// and bounded: one that runs out records BILU_ERR_TIMEOUT and every warp
-// leaves.
+// runs of 32 rows in solve order through a ticket, a lane per row; done[j]
+// holds l(j) + 1 once known (0 = pending) and is itself the flag.  Rows outside
+// the run are waited for, all belonging to runs whose tickets were handed out
+// before; those inside it follow lane by lane in registers.  (One row per warp
+// had 9.7 k rows in flight, 2.4 planes of a 64x64x32 grid whose wavefront spans
+// all of it: 1.27 ms a triangle.)  The waits are warp-uniform and bounded: one
+// that runs out records BILU_ERR_TIMEOUT and every warp leaves.
 template <bool UPPER>
-__global__ void __launch_bounds__(256) eq4_level_kernel(int32_t n, const int32_t* __restrict__ rpv,
+__global__ void __launch_bounds__(128) eq4_level_kernel(int32_t n, const int32_t* __restrict__ rpv,
                                                         const int32_t* __restrict__ civ, int32_t* done,
                                                         int32_t* __restrict__ lvl, int32_t* header, int32_t* stats,
                                                         long long spin_ns) {
   const int lane = threadIdx.x & 31;
+  const int runs = (n + 31) / 32;
   Waiter w{header, spin_ns, 0, nullptr};
+  int top = 0;
   for (;;) {
     int tk = 0;
     if (lane == 0) {
       tk = atomicAdd(header + (UPPER ? kTicketU : kTicketL), 1);
-      if (ld_volatile_s32(header + kAbort)) tk = n;
+      if (ld_volatile_s32(header + kAbort)) tk = runs;
     }
     tk = __shfl_sync(kFull, tk, 0);
-    if (tk >= n) return;
-    const int i = UPPER ? n - 1 - tk : tk;
-    const int beg = rpv[i], end = rpv[i + 1];
-    int m = 0;
-    bool ok = true;
-    for (int t0 = beg; t0 < end && ok; t0 += 32) {
-      const int t = t0 + lane;
-      const bool has = t < end;
-      const int j = has ? civ[t] : i;
-      int v = has ? ld_relaxed_s32(done + j) : 1;
-      w.t0 = 0;
-      for (unsigned it = 1;; ++it) {
-        if (__all_sync(kFull, v != 0)) break;
-        if ((it & 31u) == 0u && __any_sync(kFull, w.give_up(0u, 0u))) {
-          ok = false;
-          break;
+    if (tk >= runs) break;
+    const int at = tk * 32 + lane;  // in solve order
+    const int i = UPPER ? n - 1 - at : at;
+    const bool has = at < n;
+    int t = has ? rpv[i] : 0;
+    const int end = has ? rpv[i + 1] : 0;
+    int m = 0;           // l(i) so far
+    unsigned inner = 0;  // dependencies inside the run: bit = lane
+    w.t0 = 0;
+    for (unsigned it = 1;; ++it) {
+      // the next dependencies, eight loads in flight; a pending one is asked for again
+      while (t < end) {
+        int v[8];  // l(j) + 1; 0: pending
+        int lane_of[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int j = t + q < end ? civ[t + q] : i;
+          lane_of[q] = (UPPER ? n - 1 - j : j) - tk * 32;
+          v[q] = t + q < end && lane_of[q] < 0 ? ld_relaxed_s32(done + j) : 1;
         }
-        const int v2 = ld_relaxed_s32(done + j);  // every lane re-reads (no per-lane branch)
-        v = v != 0 ? v : v2;
+        int got = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (got == q && t + q < end && v[q] != 0) {
+            got = q + 1;
+            if (lane_of[q] < 0) m = max(m, v[q]);
+            else inner |= 1u << lane_of[q];
+          }
+        t += got;
+        if (got < 8) break;
       }
-      m = max(m, has ? v : 0);
+      if (!__any_sync(kFull, t < end)) break;
+      if ((it & 31u) == 0u && __any_sync(kFull, w.give_up(0u, 0u))) return;  // the abort word stops every other warp
     }
-    if (!ok) return;  // the abort word stops every other warp
-    m = __reduce_max_sync(kFull, m);
-    if (lane == 0) {
+#pragma unroll 4
+    for (int q = 0; q < 31; ++q) {  // lane q is final when its turn comes
+      const int lq = __shfl_sync(kFull, m, q);
+      if ((inner >> q) & 1u) m = max(m, lq + 1);
+    }
+    if (has) {
       lvl[i] = m;
       st_relaxed_s32(done + i, m + 1);
-      atomicMax(stats + (UPPER ? kNlevU : kNlevL), m + 1);
     }
+    top = max(top, __reduce_max_sync(kFull, has ? m + 1 : 0));
   }
+  if (lane == 0 && top > 0) atomicMax(stats + (UPPER ? kNlevU : kNlevL), top);
 }
 
 // Backfill gather map (Algorithm 5 steps 3-4): the factor slot of every block
@@ -442,81 +684,122 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
                                  int32_t row_capacity, void* stream, bilu_pattern** out) {
   if (!out || k < 0 || row_capacity < 1 || row_capacity > 8192) return BILU_ERR_ARG;
   *out = nullptr;
-  const int st0 = validate_pattern(n, row_ptr, col_idx);
-  if (st0 != BILU_OK) return st0;
+  if (n < 0) return BILU_ERR_ARG;
   if (n == 0) return bilu_symbolic(n, row_ptr, col_idx, k, out);
+  if (!row_ptr || (row_ptr[n] > 0 && !col_idx)) return BILU_ERR_ARG;
+  if (row_ptr[0] != 0 || row_ptr[n] < n) return BILU_ERR_PATTERN;  // each row holds its diagonal
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t nnz_a = row_ptr[n];
   const int cap = row_capacity;
-  DevBuf d_arp, d_aci, d_ocol, d_olev, d_olen, d_done, d_header;
-  if (!d_arp.alloc(sizeof(int32_t) * ((size_t)n + 1)) || !d_aci.alloc(sizeof(int32_t) * (size_t)nnz_a) ||
-      !d_ocol.alloc(sizeof(int32_t) * (size_t)n * cap) || !d_olev.alloc(sizeof(int32_t) * (size_t)n * cap) ||
-      !d_olen.alloc(sizeof(int32_t) * (size_t)n) || !d_done.alloc(sizeof(int32_t) * (size_t)n) ||
-      !d_header.alloc(kHeaderBytes)) {
-    cudaGetLastError();
-    return BILU_ERR_OOM;
-  }
-  int32_t hdr[kHeaderWords] = {};
-  hdr[kBadRow] = INT_MAX;
-  cudaMemcpyAsync(d_arp.p, row_ptr, sizeof(int32_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(d_aci.p, col_idx, sizeof(int32_t) * (size_t)nnz_a, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(d_header.p, hdr, sizeof(hdr), cudaMemcpyHostToDevice, s);
-  cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
-  const size_t smem = (size_t)kSymWarps * (4 * (size_t)cap + 32) * sizeof(int);
-  if (smem > 227 * 1024) return BILU_ERR_ARG;
-  cudaFuncSetAttribute(symbolic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)std::max<size_t>(smem, 48 * 1024));
-  int dev = 0, sms = 1, per_sm = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, symbolic_kernel, kSymWarps * 32, smem);
-  const int grid = (int)std::max<long long>(1, std::min<long long>((n + kSymWarps - 1) / kSymWarps,
-                                                                    (long long)std::max(per_sm, 1) * sms));
-  {
-    ProfScope ps(BILU_PROF_SYMBOLIC, stream);
-    symbolic_kernel<<<grid, kSymWarps * 32, smem, s>>>(n, k, cap, d_arp.as<int32_t>(), d_aci.as<int32_t>(),
-                                                       d_ocol.as<int32_t>(), d_olev.as<int32_t>(),
-                                                       d_olen.as<int32_t>(), d_done.as<int32_t>(),
-                                                       d_header.as<int32_t>(), trisolve_config().spin_ns);
-  }
-  if (cudaGetLastError() != cudaSuccess) return BILU_ERR_CUDA;
-  if (cudaMemcpyAsync(hdr, d_header.p, sizeof(hdr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    return BILU_ERR_CUDA;
-  if (hdr[kErr]) return hdr[kErr];
-  // ---- completion on the device: row pointers, L / U' split, Eq. 4 levels,
-  // backfill map, line length -- into the handle's device copy ----
+  const size_t merge_smem = (size_t)kSymWarps * (4 * (size_t)cap + 32) * sizeof(int);
+  const bool cap_fits = merge_smem <= 227 * 1024;
   const long long ntiles = ((long long)n + kScanTile - 1) / kScanTile;
-  const int gsm = std::max(1, sms * 8);
-  DevBuf d_nl, d_nu, d_flag, d_part, d_stats, d_rp0, d_lrp0, d_urp0, d_idx, d_starts, d_hist;
-  if (!d_nl.alloc(sizeof(int32_t) * (size_t)n) || !d_nu.alloc(sizeof(int32_t) * (size_t)n) ||
-      !d_flag.alloc(sizeof(int32_t) * (size_t)n) || !d_part.alloc(sizeof(long long) * (size_t)(ntiles + 1)) ||
-      !d_stats.alloc(sizeof(int32_t) * kStatWords) || !d_rp0.alloc(sizeof(int32_t) * ((size_t)n + 1)) ||
-      !d_lrp0.alloc(sizeof(int32_t) * ((size_t)n + 1)) || !d_urp0.alloc(sizeof(int32_t) * ((size_t)n + 1)) ||
-      !d_idx.alloc(sizeof(int32_t) * ((size_t)n + 1)) || !d_starts.alloc(sizeof(int32_t) * (size_t)n) ||
+  DevBuf d_arp, d_aci, d_olen, d_done, d_header, d_nl, d_nu, d_flag, d_part, d_stats, d_rp0, d_lrp0, d_urp0, d_idx,
+      d_starts, d_hist;
+  const size_t rows = sizeof(int32_t) * (size_t)n, rows1 = sizeof(int32_t) * ((size_t)n + 1);
+  if (!d_arp.alloc(rows1) || !d_aci.alloc(sizeof(int32_t) * (size_t)nnz_a) || !d_olen.alloc(rows) ||
+      !d_done.alloc(rows) || !d_header.alloc(kHeaderBytes) || !d_nl.alloc(rows) || !d_nu.alloc(rows) ||
+      !d_flag.alloc(rows) || !d_part.alloc(4 * sizeof(long long) * (size_t)(ntiles + 1)) ||
+      !d_stats.alloc(sizeof(int32_t) * kStatWords) || !d_rp0.alloc(rows1) || !d_lrp0.alloc(rows1) ||
+      !d_urp0.alloc(rows1) || !d_idx.alloc(rows1) || !d_starts.alloc(rows) ||
       !d_hist.alloc(sizeof(int32_t) * 4097)) {
     cudaGetLastError();
     return BILU_ERR_OOM;
   }
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int gsm = std::max(1, sms * 8);
+  int32_t hdr[kHeaderWords] = {};
+  hdr[kBadRow] = INT_MAX;
+  int32_t stats[kStatWords] = {};
+  cudaMemcpyAsync(d_arp.p, row_ptr, rows1, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(d_aci.p, col_idx, sizeof(int32_t) * (size_t)nnz_a, cudaMemcpyHostToDevice, s);
+  cudaMemcpyAsync(d_header.p, hdr, sizeof(hdr), cudaMemcpyHostToDevice, s);
   cudaMemsetAsync(d_stats.p, 0, sizeof(int32_t) * kStatWords, s);
   cudaMemsetAsync(d_hist.p, 0, sizeof(int32_t) * 4097, s);
-  row_info_kernel<<<gsm, 256, 0, s>>>(n, cap, d_ocol.as<int32_t>(), d_olen.as<int32_t>(), d_nl.as<int32_t>(),
-                                      d_nu.as<int32_t>(), d_flag.as<int32_t>(), d_stats.as<int32_t>());
-  // exclusive scans; the totals are checked against the int32 range
-  auto exscan = [&](const int32_t* in, int32_t* outp, long long* total) -> bool {
-    scan_tiles_kernel<<<(unsigned)ntiles, kScanTile, 0, s>>>(in, n, outp, d_part.as<long long>());
-    scan_parts_kernel<<<1, kScanTile, 0, s>>>(d_part.as<long long>(), ntiles);
-    scan_add_kernel<<<(unsigned)(((long long)n + 256) / 256), 256, 0, s>>>(outp, n, d_part.as<long long>(), ntiles);
-    return cudaMemcpyAsync(total, d_part.as<long long>() + ntiles, sizeof(long long), cudaMemcpyDeviceToHost, s) ==
-               cudaSuccess &&
-           cudaStreamSynchronize(s) == cudaSuccess;
-  };
-  long long nnz_p = 0, nnz_l = 0, nnz_u = 0, nstarts = 0;
-  if (!exscan(d_olen.as<int32_t>(), d_rp0.as<int32_t>(), &nnz_p) ||
-      !exscan(d_nl.as<int32_t>(), d_lrp0.as<int32_t>(), &nnz_l) ||
-      !exscan(d_nu.as<int32_t>(), d_urp0.as<int32_t>(), &nnz_u) ||
-      !exscan(d_flag.as<int32_t>(), d_idx.as<int32_t>(), &nstarts))
+  check_kernel<<<gsm, 256, 0, s>>>(n, (int32_t)nnz_a, d_arp.as<int32_t>(), d_aci.as<int32_t>(),
+                                   d_stats.as<int32_t>() + kBadPattern, d_stats.as<int32_t>() + kLongest);
+  if (cudaMemcpyAsync(stats, d_stats.p, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
     return BILU_ERR_CUDA;
+  if (stats[kBadPattern]) return BILU_ERR_PATTERN;
+  if (!cap_fits) return BILU_ERR_ARG;
+  // ---- rows of P': by paths (counted here, written once the sizes are
+  // known), the smaller table for short rows; by merges where they do not fit ----
+  DevBuf d_ocol, d_olev;  // the merges' rows
+  auto run_paths = [&](bool small, bool emit, const int32_t* rp, const int32_t* lrp, const int32_t* urp,
+                       long long nnz_l, int32_t* ci, int32_t* lev, int32_t* lci, int32_t* uci, int32_t* slot) {
+    auto launch = [&](auto kernel, int ints) {
+      const int smem = kPathWarps * ints * (int)sizeof(int);
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      int per_sm = 1;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPathWarps * 32, smem);
+      const int grid = (int)std::max<long long>(1, std::min<long long>((n + kPathWarps - 1) / kPathWarps,
+                                                                       (long long)std::max(per_sm, 1) * sms));
+      ProfScope ps(BILU_PROF_SYMBOLIC, stream);
+      kernel<<<grid, kPathWarps * 32, smem, s>>>(n, k, cap, emit, d_arp.as<int32_t>(), d_aci.as<int32_t>(),
+                                                 d_olen.as<int32_t>(), d_nl.as<int32_t>(), d_nu.as<int32_t>(),
+                                                 d_flag.as<int32_t>(), d_stats.as<int32_t>(), rp, lrp, urp, nnz_l, ci,
+                                                 lev, lci, uci, slot, d_header.as<int32_t>());
+    };
+    if (small) launch(path_kernel<128, 8>, PathTable<128>::kInts);
+    else launch(path_kernel<512, 32>, PathTable<512>::kInts);
+  };
+  auto read_header = [&]() {
+    return cudaMemcpyAsync(hdr, d_header.p, sizeof(hdr), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+           cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+  };
+  bool paths = false, small = stats[kLongest] <= 8;
+  for (int attempt = 0; k <= kMaxPathLevel && attempt < 2 && !paths; ++attempt) {
+    run_paths(small, false, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
+    if (!read_header()) return BILU_ERR_CUDA;
+    paths = hdr[kErr] == 0;
+    if (!paths) {
+      cudaMemsetAsync(d_header.as<int32_t>() + kErr, 0, sizeof(int32_t), s);
+      cudaMemsetAsync(d_stats.p, 0, sizeof(int32_t) * kStatWords, s);
+      if (!small) break;
+      small = false;
+    }
+  }
+  if (!paths) {
+    if (!d_ocol.alloc(rows * cap) || !d_olev.alloc(rows * cap)) {
+      cudaGetLastError();
+      return BILU_ERR_OOM;
+    }
+    cudaMemsetAsync(d_done.p, 0, rows, s);
+    cudaFuncSetAttribute(symbolic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)std::max<size_t>(merge_smem, 48 * 1024));
+    int per_sm = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, symbolic_kernel, kSymWarps * 32, merge_smem);
+    const int grid = (int)std::max<long long>(1, std::min<long long>((n + kSymWarps - 1) / kSymWarps,
+                                                                      (long long)std::max(per_sm, 1) * sms));
+    {
+      ProfScope ps(BILU_PROF_SYMBOLIC, stream);
+      symbolic_kernel<<<grid, kSymWarps * 32, merge_smem, s>>>(
+          n, k, cap, d_arp.as<int32_t>(), d_aci.as<int32_t>(), d_ocol.as<int32_t>(), d_olev.as<int32_t>(),
+          d_olen.as<int32_t>(), d_done.as<int32_t>(), d_header.as<int32_t>(), trisolve_config().spin_ns);
+    }
+    if (!read_header()) return BILU_ERR_CUDA;
+    if (hdr[kErr]) return hdr[kErr];
+    row_info_kernel<<<gsm, 256, 0, s>>>(n, cap, d_ocol.as<int32_t>(), d_olen.as<int32_t>(), d_nl.as<int32_t>(),
+                                        d_nu.as<int32_t>(), d_flag.as<int32_t>(), d_stats.as<int32_t>());
+  }
+  // ---- completion on the device: row pointers, L / U' split, Eq. 4 levels,
+  // backfill map, line length -- into the handle's device copy ----
+  // exclusive scans; the totals are checked against the int32 range
+  long long totals[4] = {0, 0, 0, 0};
+  auto exscan = [&](int q, const DevBuf& in, const DevBuf& outp) -> bool {
+    long long* const part = d_part.as<long long>() + q * (ntiles + 1);
+    scan_tiles_kernel<<<(unsigned)ntiles, kScanTile, 0, s>>>(in.as<int32_t>(), n, outp.as<int32_t>(), part);
+    scan_parts_kernel<<<1, kScanTile, 0, s>>>(part, ntiles);
+    scan_add_kernel<<<(unsigned)(((long long)n + 256) / 256), 256, 0, s>>>(outp.as<int32_t>(), n, part, ntiles);
+    return cudaMemcpyAsync(totals + q, part + ntiles, sizeof(long long), cudaMemcpyDeviceToHost, s) == cudaSuccess;
+  };
+  if (!exscan(0, d_olen, d_rp0) || !exscan(1, d_nl, d_lrp0) || !exscan(2, d_nu, d_urp0) ||
+      !exscan(3, d_flag, d_idx) || cudaStreamSynchronize(s) != cudaSuccess)
+    return BILU_ERR_CUDA;
+  const long long nnz_p = totals[0], nnz_l = totals[1], nnz_u = totals[2], nstarts = totals[3];
   if (nnz_p > (long long)INT32_MAX || nnz_l + n + nnz_u > (long long)INT32_MAX) return BILU_ERR_OOM;
   const long long nslots = nnz_l + n + nnz_u;
   // the handle's device copies: P' and its levels (d_sym), and the layout the
@@ -552,27 +835,30 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   cudaMemcpyAsync(d_rp, d_rp0.p, rpb, cudaMemcpyDeviceToDevice, s);
   cudaMemcpyAsync(d_lrp, d_lrp0.p, rpb, cudaMemcpyDeviceToDevice, s);
   cudaMemcpyAsync(d_urp, d_urp0.p, rpb, cudaMemcpyDeviceToDevice, s);
-  split_kernel<<<gsm, 256, 0, s>>>(n, cap, d_ocol.as<int32_t>(), d_olev.as<int32_t>(), d_rp, d_lrp, d_urp, d_ci,
-                                   d_lev, d_lci, d_uci);
-  cudaMemsetAsync(d_slot, 0xFF, sizeof(int32_t) * (size_t)nslots, s);
-  slot_map_kernel<<<gsm, 256, 0, s>>>(n, d_arp.as<int32_t>(), d_aci.as<int32_t>(), d_rp, d_ci, d_lrp, d_urp, nnz_l,
-                                      d_slot);
-  // Eq. 4, lower then upper: persistent grids, one warp per claimed row
+  if (paths) {
+    run_paths(small, true, d_rp, d_lrp, d_urp, nnz_l, d_ci, d_lev, d_lci, d_uci, d_slot);
+  } else {
+    split_kernel<<<gsm, 256, 0, s>>>(n, cap, d_ocol.as<int32_t>(), d_olev.as<int32_t>(), d_rp, d_lrp, d_urp, d_ci,
+                                     d_lev, d_lci, d_uci);
+    cudaMemsetAsync(d_slot, 0xFF, sizeof(int32_t) * (size_t)nslots, s);
+    slot_map_kernel<<<gsm, 256, 0, s>>>(n, d_arp.as<int32_t>(), d_aci.as<int32_t>(), d_rp, d_ci, d_lrp, d_urp, nnz_l,
+                                        d_slot);
+  }
+  // Eq. 4, lower then upper: persistent grids, one warp per claimed run of 32 rows
   int lv_per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lv_per_sm, eq4_level_kernel<false>, 256, 0);
-  const int lgrid = std::max(1, std::min<int>((n + 7) / 8, std::max(lv_per_sm, 1) * sms));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lv_per_sm, eq4_level_kernel<false>, 128, 0);
+  const int lgrid = std::max(1, std::min<int>((n + 127) / 128, std::max(lv_per_sm, 1) * sms));
   cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
-  eq4_level_kernel<false><<<lgrid, 256, 0, s>>>(n, d_lrp, d_lci, d_done.as<int32_t>(), d_lvl_l,
+  eq4_level_kernel<false><<<lgrid, 128, 0, s>>>(n, d_lrp, d_lci, d_done.as<int32_t>(), d_lvl_l,
                                                  d_header.as<int32_t>(), d_stats.as<int32_t>(),
                                                  trisolve_config().spin_ns);
   cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
-  eq4_level_kernel<true><<<lgrid, 256, 0, s>>>(n, d_urp, d_uci, d_done.as<int32_t>(), d_lvl_u,
+  eq4_level_kernel<true><<<lgrid, 128, 0, s>>>(n, d_urp, d_uci, d_done.as<int32_t>(), d_lvl_u,
                                                 d_header.as<int32_t>(), d_stats.as<int32_t>(),
                                                 trisolve_config().spin_ns);
   // line length
   line_starts_kernel<<<gsm, 256, 0, s>>>(n, d_flag.as<int32_t>(), d_idx.as<int32_t>(), d_starts.as<int32_t>());
   line_hist_kernel<<<gsm, 256, 0, s>>>((int32_t)nstarts, d_starts.as<int32_t>(), d_hist.as<int32_t>());
-  int32_t stats[kStatWords] = {};
   std::vector<int32_t> hist(4097, 0);
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(stats, d_stats.p, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
