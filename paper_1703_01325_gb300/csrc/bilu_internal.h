@@ -168,7 +168,8 @@ size_t apply_workspace_bytes(int32_t n, int32_t b);
 // Builds (host) and uploads schedule *s for `chunk` rows per chunk (the U'
 // part only if `upper`).  Allocates device memory and synchronises; the
 // previous schedule is freed only once the new one is in place.
-int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper);
+struct RowGaps;
+int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, RowGaps* gaps);
 // Host part (symbolic.cpp).
 void build_schedule(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
 // The parts of a schedule both builders share (symbolic.cpp): chunk cuts from
@@ -183,7 +184,11 @@ void ticket_order_lists(int32_t nchunks, const std::vector<int32_t>& prio, const
 // Device part for patterns completed on the device (schedule_gpu.cu): the same
 // schedule as build_schedule, with every pass over P' run on the device; it
 // allocates and fills s->d_mem (ord on the device only).
-int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
+struct RowGaps {  // of one pattern, for the schedules built from it in one call (empty: not read yet)
+  std::vector<int32_t> l, u;
+};
+int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s,
+                          RowGaps* gaps = nullptr);
 // Eq. 4 levels, L / U' split and backfill map of a pattern with rp, ci, lev set.
 int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col_idx);
 // Fills the host vectors of a device-built pattern from its device copies

@@ -542,11 +542,11 @@ void free_schedule(bilu_chunk_schedule* s) {
   s->chunk = 0;
 }
 
-int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper) {
+int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, RowGaps* gaps) {
   bilu_chunk_schedule t;
   if (!p->host_ready) {
     // completed on the device: every pass over P' on the device too
-    const int st = build_schedule_device(p, chunk, upper, &t);
+    const int st = build_schedule_device(p, chunk, upper, &t, gaps);
     if (st != BILU_OK) return (int)cudaErrorMemoryAllocation;
     free_schedule(s);
     *s = std::move(t);
