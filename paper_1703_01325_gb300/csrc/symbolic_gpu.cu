@@ -547,7 +547,7 @@ __device__ __forceinline__ void st_relaxed_s32(int32_t* p, int v) {
 // runs of 32 rows in solve order through a ticket, a lane per row; done[j]
 // holds l(j) + 1 once known (0 = pending) and is itself the flag.  Rows outside
 // the run are waited for, all belonging to runs whose tickets were handed out
-// before; those inside it follow lane by lane in registers.  (One row per warp
+// before; those inside it hand on their level in registers.  (One row per warp
 // had 9.7 k rows in flight, 2.4 planes of a 64x64x32 grid whose wavefront spans
 // all of it: 1.27 ms a triangle.)  The waits are warp-uniform and bounded: one
 // that runs out records BILU_ERR_TIMEOUT and every warp leaves.
@@ -574,41 +574,55 @@ __global__ void __launch_bounds__(128) eq4_level_kernel(int32_t n, const int32_t
     int t = has ? rpv[i] : 0;
     const int end = has ? rpv[i + 1] : 0;
     int m = 0;           // l(i) so far
-    unsigned inner = 0;  // dependencies inside the run: bit = lane
+    unsigned inner = 0;  // dependencies inside the run not done yet: bit = lane
+    for (int u = t; u < end; ++u) {
+      const int j = civ[u];
+      const int at_j = (UPPER ? n - 1 - j : j) - tk * 32;
+      if (at_j >= 0) inner |= 1u << at_j;
+    }
+    bool fin = !has;
     w.t0 = 0;
     for (unsigned it = 1;; ++it) {
-      // the next dependencies, eight loads in flight; a pending one is asked for again
+      // the next dependencies outside, eight loads in flight; a pending one is asked for again
       while (t < end) {
-        int v[8];  // l(j) + 1; 0: pending
-        int lane_of[8];
+        int v[8];  // l(j) + 1; 0: pending; -1: inside the run
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int j = t + q < end ? civ[t + q] : i;
-          lane_of[q] = (UPPER ? n - 1 - j : j) - tk * 32;
-          v[q] = t + q < end && lane_of[q] < 0 ? ld_relaxed_s32(done + j) : 1;
+          v[q] = t + q < end && (UPPER ? n - 1 - j : j) < tk * 32 ? ld_relaxed_s32(done + j) : -1;
         }
         int got = 0;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (got == q && t + q < end && v[q] != 0) {
             got = q + 1;
-            if (lane_of[q] < 0) m = max(m, v[q]);
-            else inner |= 1u << lane_of[q];
+            m = max(m, v[q]);
           }
         t += got;
         if (got < 8) break;
       }
-      if (!__any_sync(kFull, t < end)) break;
+      // rows that have all they need are published at once (a run may hold the
+      // end of one grid line and the start of the next)
+      for (;;) {
+        const bool now = !fin && t >= end && inner == 0;
+        const unsigned done_now = __ballot_sync(kFull, now);
+        if (!done_now) break;
+        if (now) {
+          lvl[i] = m;
+          st_relaxed_s32(done + i, m + 1);
+          fin = true;
+        }
+        for (unsigned x = done_now; x; x &= x - 1) {
+          const int q = __ffs(x) - 1;
+          const int lq = __shfl_sync(kFull, m, q);
+          if ((inner >> q) & 1u) {
+            m = max(m, lq + 1);
+            inner &= ~(1u << q);
+          }
+        }
+      }
+      if (__all_sync(kFull, fin)) break;
       if ((it & 31u) == 0u && __any_sync(kFull, w.give_up(0u, 0u))) return;  // the abort word stops every other warp
-    }
-#pragma unroll 4
-    for (int q = 0; q < 31; ++q) {  // lane q is final when its turn comes
-      const int lq = __shfl_sync(kFull, m, q);
-      if ((inner >> q) & 1u) m = max(m, lq + 1);
-    }
-    if (has) {
-      lvl[i] = m;
-      st_relaxed_s32(done + i, m + 1);
     }
     top = max(top, __reduce_max_sync(kFull, has ? m + 1 : 0));
   }
