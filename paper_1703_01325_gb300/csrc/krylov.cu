@@ -15,7 +15,8 @@
 // kernel of an iteration returns at once when the device stop word is set, so
 // the host can enqueue several iterations and look at the state only between
 // batches.  Dot products reduce in two deterministic stages (fixed grid of
-// per-block partial sums, then one block), so a run is bitwise reproducible.
+// per-block partial sums, then the block that stored the last of them sums them
+// in fixed order), so a run is bitwise reproducible.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -38,6 +39,7 @@ struct KState {
   double last2;            // last squared residual norm the recurrences produced
   double true2;            // squared true residual norm (after the loop)
   int stop, reason, iters, maxit;
+  unsigned arrived;        // blocks of the running reduction that have stored their partial sums
 };
 
 __device__ __forceinline__ bool stopped(const KState* st) {
@@ -62,119 +64,15 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NV], double* part
   }
 }
 
-// r = rhs - t, r_hat = r, p = v = 0; partials: (r, r), (rhs, rhs)
-__global__ void k_init(long long m, const double* rhs, const double* t, double* r, double* rh,
-                       double* p, double* v, double* partials) {
-  double acc[2] = {0.0, 0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x) {
-    const double b = rhs[q];
-    const double rq = b - t[q];
-    r[q] = rq;
-    rh[q] = rq;
-    p[q] = 0.0;
-    v[q] = 0.0;
-    acc[0] = fma(rq, rq, acc[0]);
-    acc[1] = fma(b, b, acc[1]);
-  }
-  block_reduce_store<2>(acc, partials);
-}
-
-// p = r + beta (p - omega v)
-__global__ void k_update_p(long long m, const KState* st, const double* r, double* p,
-                           const double* v) {
-  if (stopped(st)) return;
-  const double beta = (st->rho / st->rho_prev) * (st->alpha / st->omega);
-  const double omega = st->omega;
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x)
-    p[q] = r[q] + beta * (p[q] - omega * v[q]);
-}
-
-// partial (a, c)
-__global__ void k_dot(long long m, const KState* st, const double* a, const double* c,
-                      double* partials) {
-  if (stopped(st)) return;
-  double acc[1] = {0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x)
-    acc[0] = fma(a[q], c[q], acc[0]);
-  block_reduce_store<1>(acc, partials);
-}
-
-// s = r - alpha v; x += alpha p_hat; partial (s, s)
-__global__ void k_s(long long m, const KState* st, const double* r, const double* v,
-                    const double* ph, double* s, double* x, double* partials) {
-  if (stopped(st)) return;
-  const double alpha = st->alpha;
-  double acc[1] = {0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x) {
-    const double sq = r[q] - alpha * v[q];
-    s[q] = sq;
-    x[q] += alpha * ph[q];
-    acc[0] = fma(sq, sq, acc[0]);
-  }
-  block_reduce_store<1>(acc, partials);
-}
-
-// partials (t, s), (t, t)
-__global__ void k_dot_ts(long long m, const KState* st, const double* t, const double* s,
-                         double* partials) {
-  if (stopped(st)) return;
-  double acc[2] = {0.0, 0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x) {
-    const double tq = t[q];
-    acc[0] = fma(tq, s[q], acc[0]);
-    acc[1] = fma(tq, tq, acc[1]);
-  }
-  block_reduce_store<2>(acc, partials);
-}
-
-// x += omega s_hat; r = s - omega t; partials (r, r), (r_hat, r)
-__global__ void k_xr(long long m, const KState* st, const double* sh, const double* s,
-                     const double* t, const double* rh, double* x, double* r, double* partials) {
-  if (stopped(st)) return;
-  const double omega = st->omega;
-  double acc[2] = {0.0, 0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x) {
-    x[q] += omega * sh[q];
-    const double rq = s[q] - omega * t[q];
-    r[q] = rq;
-    acc[0] = fma(rq, rq, acc[0]);
-    acc[1] = fma(rh[q], rq, acc[1]);
-  }
-  block_reduce_store<2>(acc, partials);
-}
-
-// t = rhs - t; partial (t, t)
-__global__ void k_resid(long long m, const double* rhs, double* t, double* partials) {
-  double acc[1] = {0.0};
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x) {
-    const double d = rhs[q] - t[q];
-    t[q] = d;
-    acc[0] = fma(d, d, acc[0]);
-  }
-  block_reduce_store<1>(acc, partials);
-}
-
-__global__ void k_zero(long long m, double* x) {
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
-       q += (long long)gridDim.x * blockDim.x)
-    x[q] = 0.0;
-}
-
 enum FinStep : int { kFinInit, kFinAlpha, kFinS, kFinOmega, kFinR, kFinTrue };
 
-// Sums the partials of one step (fixed order) and advances the scalar state.
-__global__ void k_fin(KState* st, const double* partials, int step, int nv, double tol) {
+// Sums the partials of one step (fixed order) and advances the scalar state;
+// run by one block of kRedThreads threads.
+__device__ void advance(KState* st, const double* partials, int step, int nv, double tol) {
   __shared__ double tot[2][kRedThreads / 32];
   double v[2] = {0.0, 0.0};
   for (int q = 0; q < nv; ++q)
-    for (int k = threadIdx.x; k < kRedBlocks; k += blockDim.x) v[q] += partials[q * kRedBlocks + k];
+    for (int k = threadIdx.x; k < kRedBlocks; k += blockDim.x) v[q] += __ldcg(partials + q * kRedBlocks + k);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int q = 0; q < 2; ++q) {
     for (int d = 16; d >= 1; d >>= 1) v[q] += __shfl_down_sync(kFull, v[q], d);
@@ -240,11 +138,138 @@ __global__ void k_fin(KState* st, const double* partials, int step, int nv, doub
   }
 }
 
+// The end of a reduction kernel: the block that stores the last partial sums
+// advances the state (a kernel of its own for that cost a launch, about 2 us,
+// after each of an iteration's five reductions).  Every block of the grid gets
+// here or, with the stop word set, none.
+template <int STEP, int NV>
+__device__ __forceinline__ void finish(KState* st, const double* partials, double tol) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&st->arrived, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x == 0) st->arrived = 0;
+  advance(st, partials, STEP, NV, tol);
+}
+
+// r = rhs - t, r_hat = r, p = v = 0; partials: (r, r), (rhs, rhs)
+__global__ void k_init(long long m, KState* st, const double* rhs, const double* t, double* r, double* rh,
+                       double* p, double* v, double* partials, double tol) {
+  double acc[2] = {0.0, 0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x) {
+    const double b = rhs[q];
+    const double rq = b - t[q];
+    r[q] = rq;
+    rh[q] = rq;
+    p[q] = 0.0;
+    v[q] = 0.0;
+    acc[0] = fma(rq, rq, acc[0]);
+    acc[1] = fma(b, b, acc[1]);
+  }
+  block_reduce_store<2>(acc, partials);
+  finish<kFinInit, 2>(st, partials, tol);
+}
+
+// p = r + beta (p - omega v)
+__global__ void k_update_p(long long m, const KState* st, const double* r, double* p,
+                           const double* v) {
+  if (stopped(st)) return;
+  const double beta = (st->rho / st->rho_prev) * (st->alpha / st->omega);
+  const double omega = st->omega;
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x)
+    p[q] = r[q] + beta * (p[q] - omega * v[q]);
+}
+
+// partial (a, c)
+__global__ void k_dot(long long m, KState* st, const double* a, const double* c, double* partials, double tol) {
+  if (stopped(st)) return;
+  double acc[1] = {0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x)
+    acc[0] = fma(a[q], c[q], acc[0]);
+  block_reduce_store<1>(acc, partials);
+  finish<kFinAlpha, 1>(st, partials, tol);
+}
+
+// s = r - alpha v; x += alpha p_hat; partial (s, s)
+__global__ void k_s(long long m, KState* st, const double* r, const double* v, const double* ph, double* s, double* x,
+                    double* partials, double tol) {
+  if (stopped(st)) return;
+  const double alpha = st->alpha;
+  double acc[1] = {0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x) {
+    const double sq = r[q] - alpha * v[q];
+    s[q] = sq;
+    x[q] += alpha * ph[q];
+    acc[0] = fma(sq, sq, acc[0]);
+  }
+  block_reduce_store<1>(acc, partials);
+  finish<kFinS, 1>(st, partials, tol);
+}
+
+// partials (t, s), (t, t)
+__global__ void k_dot_ts(long long m, KState* st, const double* t, const double* s, double* partials, double tol) {
+  if (stopped(st)) return;
+  double acc[2] = {0.0, 0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x) {
+    const double tq = t[q];
+    acc[0] = fma(tq, s[q], acc[0]);
+    acc[1] = fma(tq, tq, acc[1]);
+  }
+  block_reduce_store<2>(acc, partials);
+  finish<kFinOmega, 2>(st, partials, tol);
+}
+
+// x += omega s_hat; r = s - omega t; partials (r, r), (r_hat, r)
+__global__ void k_xr(long long m, KState* st, const double* sh, const double* s, const double* t, const double* rh,
+                     double* x, double* r, double* partials, double tol) {
+  if (stopped(st)) return;
+  const double omega = st->omega;
+  double acc[2] = {0.0, 0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x) {
+    x[q] += omega * sh[q];
+    const double rq = s[q] - omega * t[q];
+    r[q] = rq;
+    acc[0] = fma(rq, rq, acc[0]);
+    acc[1] = fma(rh[q], rq, acc[1]);
+  }
+  block_reduce_store<2>(acc, partials);
+  finish<kFinR, 2>(st, partials, tol);
+}
+
+// t = rhs - t; partial (t, t)
+__global__ void k_resid(long long m, KState* st, const double* rhs, double* t, double* partials, double tol) {
+  double acc[1] = {0.0};
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x) {
+    const double d = rhs[q] - t[q];
+    t[q] = d;
+    acc[0] = fma(d, d, acc[0]);
+  }
+  block_reduce_store<1>(acc, partials);
+  finish<kFinTrue, 1>(st, partials, tol);
+}
+
+__global__ void k_zero(long long m, double* x) {
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < m;
+       q += (long long)gridDim.x * blockDim.x)
+    x[q] = 0.0;
+}
+
 __global__ void k_state_reset(KState* st, int maxit) {
   st->iters = 0;
   st->maxit = maxit;
   st->stop = 0;
   st->reason = kRunning;
+  st->arrived = 0;
 }
 
 
@@ -340,24 +365,19 @@ int bicgstab_core(const KOps& ops, long long m, const double* rhs, double* x, do
   for (;;) {
     // (re)start from the residual of the current x
     if (ops.spmv(x, t, nullptr, awork)) { status = BILU_ERR_CUDA; break; }
-    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_init<<<vb, vt, 0, s>>>(m, rhs, t, r, rh, pv, v, partials); }
-    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinInit, 2, tol); }
+    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_init<<<vb, vt, 0, s>>>(m, st, rhs, t, r, rh, pv, v, partials, tol); }
     bool done_loop = false;
     while (!done_loop) {
       for (int it = 0; it < batch; ++it) {
         { ProfScope ps_(BILU_PROF_KRYLOV, s); k_update_p<<<vb, vt, 0, s>>>(m, st, r, pv, v); }
         ops.apply(pv, ph, stop, awork);
         spmv_applied(ph, v, stop, awork);
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_dot<<<vb, vt, 0, s>>>(m, st, rh, v, partials); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinAlpha, 1, tol); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_s<<<vb, vt, 0, s>>>(m, st, r, v, ph, sv, x, partials); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinS, 1, tol); }
+        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_dot<<<vb, vt, 0, s>>>(m, st, rh, v, partials, tol); }
+        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_s<<<vb, vt, 0, s>>>(m, st, r, v, ph, sv, x, partials, tol); }
         ops.apply(sv, sh, stop, awork);
         spmv_applied(sh, t, stop, awork);
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_dot_ts<<<vb, vt, 0, s>>>(m, st, t, sv, partials); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinOmega, 2, tol); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_xr<<<vb, vt, 0, s>>>(m, st, sh, sv, t, rh, x, r, partials); }
-        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinR, 2, tol); }
+        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_dot_ts<<<vb, vt, 0, s>>>(m, st, t, sv, partials, tol); }
+        { ProfScope ps_(BILU_PROF_KRYLOV, s); k_xr<<<vb, vt, 0, s>>>(m, st, sh, sv, t, rh, x, r, partials, tol); }
       }
       if (cudaGetLastError() != cudaSuccess) { status = BILU_ERR_CUDA; done_loop = true; break; }
       int aerr = 0;
@@ -386,8 +406,7 @@ int bicgstab_core(const KOps& ops, long long m, const double* rhs, double* x, do
     }
     // true residual
     ops.spmv(x, t, nullptr, awork);
-    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_resid<<<vb, vt, 0, s>>>(m, rhs, t, partials); }
-    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_fin<<<1, vt, 0, s>>>(st, partials, kFinTrue, 1, tol); }
+    { ProfScope ps_(BILU_PROF_KRYLOV, s); k_resid<<<vb, vt, 0, s>>>(m, st, rhs, t, partials, tol); }
     if (cudaMemcpyAsync(&hs, st, sizeof(KState), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
       status = BILU_ERR_CUDA;
