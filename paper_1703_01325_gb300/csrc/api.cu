@@ -25,9 +25,9 @@ int solve_schedule(const bilu_pattern* p) {
 int factor_schedule(const bilu_pattern* p) { return (p->n == 0 || p->fact.d_mem) ? BILU_OK : BILU_ERR_STATE; }
 
 int build_schedules(bilu_pattern* p) {
-  RowGaps gaps;
-  if (make_schedule(p, &p->solve, solve_chunk_target(p), true, &gaps) != 0) return BILU_ERR_OOM;
-  if (!p->is_transpose && make_schedule(p, &p->fact, factor_chunk_target(p), false, &gaps) != 0) return BILU_ERR_OOM;
+  ScheduleInputs in;
+  if (make_schedule(p, &p->solve, solve_chunk_target(p), true, &in) != 0) return BILU_ERR_OOM;
+  if (!p->is_transpose && make_schedule(p, &p->fact, factor_chunk_target(p), false, &in) != 0) return BILU_ERR_OOM;
   return BILU_OK;
 }
 

@@ -168,8 +168,8 @@ size_t apply_workspace_bytes(int32_t n, int32_t b);
 // Builds (host) and uploads schedule *s for `chunk` rows per chunk (the U'
 // part only if `upper`).  Allocates device memory and synchronises; the
 // previous schedule is freed only once the new one is in place.
-struct RowGaps;
-int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, RowGaps* gaps);
+struct ScheduleInputs;
+int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in);
 // Host part (symbolic.cpp).
 void build_schedule(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
 // The parts of a schedule both builders share (symbolic.cpp): chunk cuts from
@@ -181,14 +181,22 @@ void schedule_cuts(int32_t n, int32_t target, bool upper, const std::vector<int3
                    const std::vector<int32_t>& gapu, bilu_chunk_schedule* s);
 void ticket_order_lists(int32_t nchunks, const std::vector<int32_t>& prio, const std::vector<int64_t>& pred_ptr,
                         const std::vector<int32_t>& pred, std::vector<int32_t>& tick);
-// Device part for patterns completed on the device (schedule_gpu.cu): the same
+// Device part (schedule_gpu.cu), for any uploaded pattern: the same
 // schedule as build_schedule, with every pass over P' run on the device; it
 // allocates and fills s->d_mem (ord on the device only).
-struct RowGaps {  // of one pattern, for the schedules built from it in one call (empty: not read yet)
-  std::vector<int32_t> l, u;
+// What the schedules built from one pattern in one call share: the row gaps
+// (empty: not read yet) and, for a pattern completed on the host, a device copy
+// of its Eq. 4 levels (else the pattern's own).
+struct ScheduleInputs {
+  std::vector<int32_t> gapl, gapu;
+  int32_t *d_lvl_l = nullptr, *d_lvl_u = nullptr;
+  ScheduleInputs() = default;
+  ScheduleInputs(const ScheduleInputs&) = delete;
+  ~ScheduleInputs();
+  bool levels(const bilu_pattern* p);  // copies them up if need be
 };
 int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s,
-                          RowGaps* gaps = nullptr);
+                          ScheduleInputs* in = nullptr);
 // Eq. 4 levels, L / U' split and backfill map of a pattern with rp, ci, lev set.
 int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col_idx);
 // Fills the host vectors of a device-built pattern from its device copies

@@ -1,7 +1,6 @@
 // schedule_gpu.cu -- the sync-free schedules (chunk cuts, the rows of each
-// chunk by local Eq. 4 level, the chunk claim order) for a pattern completed
-// on the device by bilu_symbolic_gpu, with every pass over P' run on the
-// device.  The result is the schedule build_schedule (symbolic.cpp) builds on
+// chunk by local Eq. 4 level, the chunk claim order) of an uploaded pattern,
+// with every pass over P' run on the device.  The result is the schedule build_schedule (symbolic.cpp) builds on
 // the host, bit for bit: the host keeps only the steps whose work grows with
 // the number of rows or chunks -- the greedy chunk cuts over the per-row gaps
 // and the list scheduling over the chunk graph -- and runs them through the
@@ -269,11 +268,10 @@ int device_sms() {
 // the device, list scheduling on the host (work per chunk, not per entry).
 template <bool UPPER>
 int ticket_order_device(const bilu_pattern* p, const bilu_chunk_schedule* s, const int32_t* d_bnd,
-                        std::vector<int32_t>& tick) {
+                        const int32_t* lvl, std::vector<int32_t>& tick) {
   const int32_t nchunks = s->nchunks;
   const int32_t* rpv = UPPER ? p->d_urp : p->d_lrp;
   const int32_t* civ = UPPER ? p->d_uci : p->d_lci;
-  const int32_t* lvl = UPPER ? p->d_lvl_u : p->d_lvl_l;
   const int grid = device_sms() * 8;
   {
     Scratch few;
@@ -351,8 +349,24 @@ int ticket_order_device(const bilu_pattern* p, const bilu_chunk_schedule* s, con
 
 }  // namespace
 
+ScheduleInputs::~ScheduleInputs() { cudaFree(d_lvl_l); }
+
+bool ScheduleInputs::levels(const bilu_pattern* p) {
+  if (d_lvl_l || p->d_lvl_l) return true;
+  const size_t n = (size_t)p->n;
+  void* m = nullptr;
+  if (cudaMalloc(&m, 2 * n * sizeof(int32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  d_lvl_l = (int32_t*)m;
+  d_lvl_u = d_lvl_l + n;
+  return cudaMemcpy(d_lvl_l, p->lvl_l.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMemcpy(d_lvl_u, p->lvl_u.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+
 int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bilu_chunk_schedule* s,
-                          RowGaps* gaps) {
+                          ScheduleInputs* in) {
   const int32_t n = p->n;
   s->chunk = target;
   s->upper = upper;
@@ -363,23 +377,24 @@ int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bil
     return BILU_OK;
   }
   try {
-    RowGaps own;
-    if (!gaps) gaps = &own;
-    if (gaps->l.empty()) {
-      gaps->l.resize((size_t)n);
-      gaps->u.resize((size_t)n);
+    ScheduleInputs own;
+    if (!in) in = &own;
+    if (!in->levels(p)) return BILU_ERR_OOM;
+    if (in->gapl.empty()) {
+      in->gapl.resize((size_t)n);
+      in->gapu.resize((size_t)n);
       Scratch sc;
       int32_t* d_gl = sc.get<int32_t>((size_t)n);
       int32_t* d_gu = sc.get<int32_t>((size_t)n);
       if (!d_gl || !d_gu) return BILU_ERR_OOM;
       gap_kernel<<<device_sms() * 8, 256>>>(n, p->d_lrp, p->d_lci, p->d_urp, p->d_uci, d_gl, d_gu);
-      if (cudaMemcpy(gaps->l.data(), d_gl, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess ||
-          cudaMemcpy(gaps->u.data(), d_gu, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess) {
-        gaps->l.clear();
+      if (cudaMemcpy(in->gapl.data(), d_gl, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess ||
+          cudaMemcpy(in->gapu.data(), d_gu, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess) {
+        in->gapl.clear();
         return BILU_ERR_CUDA;
       }
     }
-    schedule_cuts(n, target, upper, gaps->l, gaps->u, s);
+    schedule_cuts(n, target, upper, in->gapl, in->gapu, s);
     if (s->max_len > kMaxChunkRows) return BILU_ERR_ARG;
     const int32_t nchunks = s->nchunks;
     const size_t one = align256(sizeof(int32_t) * (size_t)n);
@@ -405,8 +420,9 @@ int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bil
     chunk_order_kernel<false><<<ogrid, kOrderWarps * 32>>>(nchunks, s->d_bnd, p->d_lrp, p->d_lci, s->d_ord_l);
     if (upper)
       chunk_order_kernel<true><<<ogrid, kOrderWarps * 32>>>(nchunks, s->d_bnd, p->d_urp, p->d_uci, s->d_ord_u);
-    int st = ticket_order_device<false>(p, s, s->d_bnd, s->tick_l);
-    if (st == BILU_OK && upper) st = ticket_order_device<true>(p, s, s->d_bnd, s->tick_u);
+    int st = ticket_order_device<false>(p, s, s->d_bnd, in->d_lvl_l ? in->d_lvl_l : p->d_lvl_l, s->tick_l);
+    if (st == BILU_OK && upper)
+      st = ticket_order_device<true>(p, s, s->d_bnd, in->d_lvl_u ? in->d_lvl_u : p->d_lvl_u, s->tick_u);
     if (st == BILU_OK) {
       cudaMemcpy(s->d_tick_l, s->tick_l.data(), sizeof(int32_t) * (size_t)nchunks, cudaMemcpyHostToDevice);
       if (upper)
