@@ -22,8 +22,10 @@ extern "C" {
  * systems still spread over the GPU; where that hits 256 and the pattern
  * shows a line length L of 16..192 rows (the most common distance between
  * rows that do not depend on their predecessor: grid-line starts in a
- * natural ordering), 2 L instead -- two grid lines per chunk; 1 <= rows <=
- * 1024 fixes the target;
+ * natural ordering), 2 L instead -- two grid lines per chunk; below that, L
+ * where the widest row of L or U' has more than 8 blocks, and otherwise a
+ * second schedule of 2 L for rows that take one pass of a warp; 1 <= rows <=
+ * 1024 fixes the target (and leaves out the second schedule);
  * other values: BILU_ERR_ARG.  Takes effect for a pattern at its next
  * bilu_pattern_upload or bilu_pattern_schedule (the set-up calls that build
  * schedules); apply, factor and solve never rebuild one. */
@@ -50,7 +52,8 @@ int32_t bilu_get_factor_chunk(void);
  * inspection (as bilu_auto_trisolve_chunk).  Returns -1 for a NULL p. */
 int32_t bilu_auto_factor_chunk(const bilu_pattern* p);
 
-/* Warps per CTA in the triangular solves: 4 (default), 8 or 16, else
+/* Warps per CTA in the triangular solves: 4 (default; 8 for rows of 40 blocks
+ * or more that take at least four passes of a warp), 8 or 16, else
  * BILU_ERR_ARG.  More warps per chunk give each row more time to fetch its
  * operands ahead of its dependencies.  Applies to the next launch. */
 int bilu_set_trisolve_warps(int32_t warps);

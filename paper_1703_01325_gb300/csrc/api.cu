@@ -27,6 +27,9 @@ int factor_schedule(const bilu_pattern* p) { return (p->n == 0 || p->fact.d_mem)
 int build_schedules(bilu_pattern* p) {
   ScheduleInputs in;
   if (make_schedule(p, &p->solve, solve_chunk_target(p), true, &in) != 0) return BILU_ERR_OOM;
+  const int32_t pair = pair_chunk_target(p);
+  if (pair > 0 && make_schedule(p, &p->pair, pair, true, &in) != 0) return BILU_ERR_OOM;
+  if (pair == 0 || !pair_chunks_fit(p)) free_schedule(&p->pair);
   if (!p->is_transpose && make_schedule(p, &p->fact, factor_chunk_target(p), false, &in) != 0) return BILU_ERR_OOM;
   return BILU_OK;
 }
@@ -131,6 +134,7 @@ extern "C" int bilu_pattern_upload(bilu_pattern* p, void* stream) {
   }
   // the schedules live on the device of the previous upload: rebuild them here
   free_schedule(&p->solve);
+  free_schedule(&p->pair);
   free_schedule(&p->fact);
   const int32_t n = p->n;
   if (n == 0) {
@@ -193,6 +197,7 @@ extern "C" void bilu_destroy_pattern(bilu_pattern* p) {
   if (p->d_mem) cudaFree(p->d_mem);
   if (p->d_sym) cudaFree(p->d_sym);
   free_schedule(&p->solve);
+  free_schedule(&p->pair);
   free_schedule(&p->fact);
   delete p;
 }

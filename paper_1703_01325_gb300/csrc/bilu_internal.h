@@ -53,9 +53,10 @@ struct bilu_pattern {
   // buffer whose transposed block lands there.
   std::vector<int32_t> slot_src;
   bool is_transpose = false;
-  // Schedules of the triangular solves and of the factorization (L only);
-  // each has its own chunk size.
-  bilu_chunk_schedule solve, fact;
+  // Schedules of the triangular solves, of their rows of one pass where those
+  // want other chunks (pair_chunk_target; else empty) and of the factorization
+  // (L only); each has its own chunk size.
+  bilu_chunk_schedule solve, pair, fact;
   // Device copy (bilu_pattern_upload).
   int device = -1;
   void* d_mem = nullptr;
@@ -121,6 +122,8 @@ TrisolveConfig& trisolve_config();
 // 128).
 int32_t solve_chunk_target(const bilu_pattern* p);
 int32_t auto_solve_chunk_target(const bilu_pattern* p);  // the rule alone
+int32_t pair_chunk_target(const bilu_pattern* p);
+bool pair_chunks_fit(const bilu_pattern* p);  // of the built schedule
 int32_t factor_chunk_target(const bilu_pattern* p);
 int32_t auto_factor_chunk_target(const bilu_pattern* p);  // the rule alone
 

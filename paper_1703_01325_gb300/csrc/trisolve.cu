@@ -80,10 +80,35 @@ int device_sm_count() {
 // chunks through global memory; three lines lengthen each chunk's chain and
 // leave fewer chunks in flight).  The chunk cut then goes to the line start
 // nearest the target.
+// Rows of more than eight blocks on smaller grids: one line, whose level has a
+// row for one warp while the others fetch theirs (27-point 80x80x40 ILU(2) b =
+// 3: 7.3 ms with two lines, 6.1 with one; 64x64x32 ILU(1): 2.57, 2.42).
 int32_t auto_solve_chunk_target(const bilu_pattern* p) {
   const long long t = (long long)p->n / (10LL * device_sm_count());
-  if (t >= 256 && p->line_len >= 16 && p->line_len <= 192) return 2 * p->line_len;
+  if (p->line_len >= 16 && p->line_len <= 192) {
+    if (t >= 256) return 2 * p->line_len;
+    if (std::max(p->max_l, p->max_u) > 8) return p->line_len;
+  }
   return (int32_t)std::max(32LL, std::min(256LL, t));
+}
+
+// The schedule of rows that take one pass over the groups, on grids too small
+// for two lines per chunk above: 0 (none), or two lines.  Such rows are done
+// within a level of two lines, and half the hand-offs between chunks go (apply,
+// us, 1 line / 2 lines: 64x64x32 ILU(1) b = 3 523 / 488, 30x30x30 323 / 285,
+// 61x47x33 ILU(0) b = 5 310 / 293, 150x30x20 ILU(1) b = 4 465 / 394); rows of
+// two passes are not (b = 5 ILU(1) 883 / 967, b = 6 874 / 937), nor grids whose
+// few lines per plane leave chunks of three (100x9x60 ILU(0) b = 8: 379 / 405;
+// pair_chunks_fit).
+int32_t pair_chunk_target(const bilu_pattern* p) {
+  if (trisolve_config().chunk > 0 || p->line_len < 16 || p->line_len > 192 ||
+      std::max(p->max_l, p->max_u) > 8 || auto_solve_chunk_target(p) == 2 * p->line_len)
+    return 0;
+  return 2 * p->line_len;
+}
+
+bool pair_chunks_fit(const bilu_pattern* p) {
+  return p->n <= 2.1 * p->line_len * p->pair.nchunks;
 }
 
 int32_t solve_chunk_target(const bilu_pattern* p) {
@@ -458,14 +483,16 @@ void launch_tri_groups(const TriArgs<TV, RT>& a, int32_t max_blocks, size_t smem
 // L y = r (y in TV), z = D^{-1} y in place, U' x = z (x in TV: the caller's
 // vector in FP64, a workspace vector widened afterwards in FP32).
 template <int B, typename TV, int W>
-void launch_solves(const bilu_pattern* p, int chunk, int nchunks, const TV* L, const TV* Dinv,
+void launch_solves(const bilu_pattern* p, const bilu_chunk_schedule& sch, const TV* L, const TV* Dinv,
                    const TV* U, const double* r, TV* y, TV* x, int32_t* header, const TrisolveConfig& cfg,
                    int32_t* stop, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
+  const int chunk = sch.max_len;  // shared-memory rows per CTA
+  const int nchunks = sch.nchunks;
   const size_t smem = tri_smem_bytes<TV>(chunk, B);
   {
-    const TriArgs<TV, double> a{p->n, chunk, nchunks, p->solve.d_bnd, p->d_lrp, p->d_lci, L,
-                                p->solve.d_ord_l, p->solve.d_tick_l, r, y, header, cfg.spin_ns, cfg.skip_row, stop};
+    const TriArgs<TV, double> a{p->n, chunk, nchunks, sch.d_bnd, p->d_lrp, p->d_lci, L,
+                                sch.d_ord_l, sch.d_tick_l, r, y, header, cfg.spin_ns, cfg.skip_row, stop};
     ProfScope ps(BILU_PROF_LOWER, stream);
     launch_tri_groups<B, false, TV, W, double>(a, p->max_l, smem, s);
   }
@@ -479,8 +506,8 @@ void launch_solves(const bilu_pattern* p, int chunk, int nchunks, const TV* L, c
     diag_scale_kernel<B, TV><<<(unsigned)blocks, 256, 0, s>>>(p->n, Dinv, y, stop);
   }
   {
-    const TriArgs<TV, TV> a{p->n, chunk, nchunks, p->solve.d_bnd, p->d_urp, p->d_uci, U,
-                            p->solve.d_ord_u, p->solve.d_tick_u, y, x, header, cfg.spin_ns, -1, stop};
+    const TriArgs<TV, TV> a{p->n, chunk, nchunks, sch.d_bnd, p->d_urp, p->d_uci, U,
+                            sch.d_ord_u, sch.d_tick_u, y, x, header, cfg.spin_ns, -1, stop};
     ProfScope ps(BILU_PROF_UPPER, stream);
     launch_tri_groups<B, true, TV, W, TV>(a, p->max_u, smem, s);
   }
@@ -494,8 +521,8 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
   cudaStream_t s = (cudaStream_t)stream;
   const TrisolveConfig& cfg = trisolve_config();
   if (p->solve.chunk <= 0 || !p->solve.upper || !p->solve.d_mem) return (int)cudaErrorInvalidValue;
-  const int chunk = p->solve.max_len;  // shared-memory rows per CTA
-  const int nchunks = p->solve.nchunks;
+  const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
+  const bilu_chunk_schedule& sch = one_pass && p->pair.d_mem && cfg.warps == 4 ? p->pair : p->solve;
   int32_t* header = reinterpret_cast<int32_t*>(work);
   const long long m = (long long)n * b;
   // The workspace's vector region holds n*b doubles: y (FP64), or y and the
@@ -513,13 +540,20 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
     ProfScope ps(BILU_PROF_APPLY_PREP, stream);
     apply_prep_kernel<TV><<<prep_blocks, 256, 0, s>>>(y, xs, m, header, stop);
   }
+  // Rows of many passes: eight warps per CTA, so that a level's rows have been
+  // fetched when their turn comes (apply, ms, 4 / 8 warps: 27-point ILU(2) b = 2
+  // 128x128x40 6.19 / 4.87, b = 3 80x80x40 6.09 / 5.88, FP32 5.06 / 4.59).  Rows
+  // of fewer blocks or passes are not faster (27-point ILU(1) b = 3 2.42 / 2.45;
+  // 27-point ILU(2) b = 1, two passes, 1.81 / 1.86).
+  const int widest = std::max(p->max_l, p->max_u);
+  const int warps = cfg.warps == 4 && widest >= 40 && widest > 3 * groups_for(b) ? 8 : cfg.warps;
   BILU_DISPATCH_B(b, {
-    if (cfg.warps == 16)
-      launch_solves<B, TV, 16>(p, chunk, nchunks, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
-    else if (cfg.warps == 4)
-      launch_solves<B, TV, 4>(p, chunk, nchunks, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
+    if (warps == 16)
+      launch_solves<B, TV, 16>(p, sch, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
+    else if (warps == 4)
+      launch_solves<B, TV, 4>(p, sch, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
     else
-      launch_solves<B, TV, 8>(p, chunk, nchunks, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
+      launch_solves<B, TV, 8>(p, sch, L, Dinv, U, r, y, xs, header, cfg, stop, stream);
   });
   if constexpr (sizeof(TV) == 4) {
     ProfScope ps(BILU_PROF_APPLY_PREP, stream);
