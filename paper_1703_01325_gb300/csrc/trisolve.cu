@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(256) widen_kernel(const float* __restrict__ sr
 // GE: the groups a row's blocks are spread over (a power of two, at most
 // groups_for(B)); the partial sums take log2(GE) reduction steps.  RT: the
 // type of the right-hand side (double r for L, TV z for U').
-template <int B, bool UPPER, typename TV, int kTriWarps, int GE, typename RT, bool DEEP>
+template <int B, bool UPPER, typename TV, int kTriWarps, int GE, typename RT, bool DEEP, bool JOIN>
 __global__ void __launch_bounds__(kTriWarps * 32) tri_solve_kernel(
     int32_t n, int32_t chunk, int32_t nchunks, const int32_t* __restrict__ bnd, const int32_t* __restrict__ rp,
     const int32_t* __restrict__ ci, const TV* __restrict__ vals,
@@ -331,9 +331,10 @@ __global__ void __launch_bounds__(kTriWarps * 32) tri_solve_kernel(
       TV acc = lane < B ? (TV)cur.own : TV(0);
       for (int t0 = cur.beg; t0 < cur.end; t0 += G) {
         const int t = t0 + g;
-        if (act && t < cur.end) {
+        const bool use = act && t < cur.end;
+        TV yt[B], av[B];
+        if (use) {
           int j;
-          TV av[B];
           typename VB::U yv[B];
           if (t0 == cur.beg) {
             j = cur.j;
@@ -351,7 +352,6 @@ __global__ void __launch_bounds__(kTriWarps * 32) tri_solve_kernel(
               yv[q] = VB::kPend;
             }
           }
-          TV yt[B];
           if (j >= lo && j < hi) {
             ok = wait_values_shared<B, TV>(yl + (size_t)(j - lo) * B, yt, w);
           } else {
@@ -363,13 +363,26 @@ __global__ void __launch_bounds__(kTriWarps * 32) tri_solve_kernel(
             }
             if (!have) ok = wait_values_global<B, TV>(out + (size_t)j * B, yt, w);
           }
-          if (ok) {
+          if constexpr (!JOIN) {
+            if (ok) {
+#pragma unroll
+              for (int q = 0; q < B; ++q) acc = fma(-av[q], yt[q], acc);
+            }
+          }
+        }
+        if constexpr (JOIN) {
+          // the lanes' waits end apart; from here the warp is whole again
+          if (__any_sync(kFull, !ok)) {
+            dead = true;
+            break;
+          }
+          if (use) {
 #pragma unroll
             for (int q = 0; q < B; ++q) acc = fma(-av[q], yt[q], acc);
           }
         }
       }
-      if (__any_sync(kFull, !ok)) {
+      if (dead || (!JOIN && __any_sync(kFull, !ok))) {
         dead = true;
         break;
       }
@@ -409,15 +422,15 @@ size_t tri_smem_bytes(int chunk, int b) {
 // Persistent grid: as many CTAs as fit on the device at once (cached per
 // shared-memory size; the occupancy query is host work worth skipping per
 // launch).
-template <int B, bool UPPER, typename TV, int kTriWarps, int GE, typename RT, bool DEEP>
+template <int B, bool UPPER, typename TV, int kTriWarps, int GE, typename RT, bool DEEP, bool JOIN>
 int tri_grid(size_t smem, int nchunks) {
   static size_t last_smem = 0;
   static int last_per_sm = 1;
   if (smem != last_smem) {
-    cudaFuncSetAttribute(tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP>,
+    cudaFuncSetAttribute(tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP, JOIN>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP>,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP, JOIN>,
                                                   kTriWarps * 32, smem);
     last_per_sm = per_sm < 1 ? 1 : per_sm;
     last_smem = smem;
@@ -442,10 +455,10 @@ struct TriArgs {
   int32_t* stop;
 };
 
-template <int B, bool UPPER, typename TV, int W, int GE, typename RT, bool DEEP>
+template <int B, bool UPPER, typename TV, int W, int GE, typename RT, bool DEEP, bool JOIN>
 void launch_tri_k(const TriArgs<TV, RT>& a, size_t smem, cudaStream_t s) {
-  const int grid = tri_grid<B, UPPER, TV, W, GE, RT, DEEP>(smem, a.nchunks);
-  tri_solve_kernel<B, UPPER, TV, W, GE, RT, DEEP><<<grid, W * 32, smem, s>>>(
+  const int grid = tri_grid<B, UPPER, TV, W, GE, RT, DEEP, JOIN>(smem, a.nchunks);
+  tri_solve_kernel<B, UPPER, TV, W, GE, RT, DEEP, JOIN><<<grid, W * 32, smem, s>>>(
       a.n, a.chunk, a.nchunks, a.bnd, a.rp, a.ci, a.vals, a.ord, a.tick, a.rhs, a.out, a.header, a.spin_ns,
       a.skip_row, a.stop);
 }
@@ -458,11 +471,31 @@ void launch_tri_k(const TriArgs<TV, RT>& a, size_t smem, cudaStream_t s) {
 // fits in one pass over the groups (FP32) or four (FP64).  Wider rows keep
 // two rows in registers: FP32 b = 6 with 2-4 passes is 20-29 % slower, FP32
 // b = 8 with 2 passes 6 %, FP64 27-point ILU(2) with 7 passes 29 %.
+//
+// JOIN: the warp is brought together after the waits of every pass and the FMAs
+// run once for all its lanes; without it lanes that waited in shared memory,
+// in global memory or not at all run theirs apart, each a pass of the FP64 pipe.
+// Measured without / with (apply, us, FP64): 96x96x48 ILU(2) b = 4 (two passes)
+// 2451 / 1862, 61x47x33 the same rows 1304 / 994, 50x45x30 ILU(1) b = 6 874 /
+// 707, 40x40x20 ILU(2) b = 8 (three) 1482 / 1234, 27-point 64x64x32 ILU(1) b = 3
+// (four) 2420 / 2111, 128x128x64 ILU(1) b = 3 (one) 1254 / 1246.  In rows of more
+// passes, or four with eight warps per CTA, a wait then holds up the loads of
+// the other lanes' next pass (27-point ILU(2): b = 3 5871 / 6962, b = 2 4676 /
+// 5373), and so it does in FP32 rows of several passes over eight or more
+// groups (b = 4 ILU(2) 849 / 884; b = 5 ILU(1) 551 / 504, b = 8 ILU(2) 1113 / 917).
 template <int B, bool UPPER, typename TV, int W, int GE, typename RT>
 void launch_tri(const TriArgs<TV, RT>& a, int32_t max_blocks, size_t smem, cudaStream_t s) {
   const int passes = (max_blocks + GE - 1) / GE;
-  if (passes > (sizeof(TV) == 4 ? 1 : 4)) launch_tri_k<B, UPPER, TV, W, GE, RT, true>(a, smem, s);
-  else launch_tri_k<B, UPPER, TV, W, GE, RT, false>(a, smem, s);
+  const bool join = passes <= (W == 4 ? 4 : 3);
+  if constexpr (sizeof(TV) == 8) {
+    if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
+    if (passes <= 4) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, false>(a, smem, s);
+  } else {
+    if (passes == 1) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
+    if constexpr (B >= 5)
+      if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, true, true>(a, smem, s);
+  }
+  launch_tri_k<B, UPPER, TV, W, GE, RT, true, false>(a, smem, s);
 }
 
 // The fewest groups (a power of two, at least groups_for(B) / 4) that hold
