@@ -99,10 +99,15 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // 61x47x33 ILU(0) b = 5 310 / 293, 150x30x20 ILU(1) b = 4 465 / 394); rows of
 // two passes are not (b = 5 ILU(1) 883 / 967, b = 6 874 / 937), nor grids whose
 // few lines per plane leave chunks of three (100x9x60 ILU(0) b = 8: 379 / 405;
-// pair_chunks_fit).
+// pair_chunks_fit).  Two long lines hold a chunk too long where a row is quick:
+// beyond kPairLine only FP64 rows of more than four blocks (FP32 105x21x9 ILU(0)
+// b = 4: 142 / 164; FP64 100x9x60 ILU(1) b = 3: 521 / 472).
+constexpr int kPairLine = 64;
+
 int32_t pair_chunk_target(const bilu_pattern* p) {
-  if (trisolve_config().chunk > 0 || p->line_len < 16 || p->line_len > 192 ||
-      std::max(p->max_l, p->max_u) > 8 || auto_solve_chunk_target(p) == 2 * p->line_len)
+  const int widest = std::max(p->max_l, p->max_u);
+  if (trisolve_config().chunk > 0 || p->line_len < 16 || p->line_len > 192 || widest > 8 ||
+      (p->line_len > kPairLine && widest <= 4) || auto_solve_chunk_target(p) == 2 * p->line_len)
     return 0;
   return 2 * p->line_len;
 }
@@ -555,7 +560,8 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
   const TrisolveConfig& cfg = trisolve_config();
   if (p->solve.chunk <= 0 || !p->solve.upper || !p->solve.d_mem) return (int)cudaErrorInvalidValue;
   const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
-  const bilu_chunk_schedule& sch = one_pass && p->pair.d_mem && cfg.warps == 4 ? p->pair : p->solve;
+  const bool lines = sizeof(TV) == 8 || p->line_len <= kPairLine;
+  const bilu_chunk_schedule& sch = one_pass && lines && p->pair.d_mem && cfg.warps == 4 ? p->pair : p->solve;
   int32_t* header = reinterpret_cast<int32_t*>(work);
   const long long m = (long long)n * b;
   // The workspace's vector region holds n*b doubles: y (FP64), or y and the
