@@ -544,15 +544,68 @@ __device__ __forceinline__ void st_relaxed_s32(int32_t* p, int v) {
 // Eq. 4 on the device: l(i) = 1 + max l(j) over the dependencies j of row i
 // (0 for a row without any), 0-based, for L (j < i, rows ascending) or for
 // the reversed graph of U' (j > i, rows descending).  Sync-free: warps claim
-// runs of 32 rows in solve order through a ticket, a lane per row; done[j]
-// holds l(j) + 1 once known (0 = pending) and is itself the flag.  Rows outside
-// the run are waited for, all belonging to runs whose tickets were handed out
-// before; those inside it hand on their level in registers.  (One row per warp
-// had 9.7 k rows in flight, 2.4 planes of a 64x64x32 grid whose wavefront spans
-// all of it: 1.27 ms a triangle.)  The waits are warp-uniform and bounded: one
-// that runs out records BILU_ERR_TIMEOUT and every warp leaves.
+// rows in solve order through a ticket, so a row only waits on rows whose
+// tickets were handed out before, all held by running warps; done[j] holds
+// l(j) + 1 once known (0 = pending) and is itself the flag.  The waits are
+// warp-uniform (the whole warp re-reads until no lane sees a pending value)
+// and bounded: one that runs out records BILU_ERR_TIMEOUT and every warp
+// leaves.
 template <bool UPPER>
-__global__ void __launch_bounds__(128) eq4_level_kernel(int32_t n, const int32_t* __restrict__ rpv,
+__global__ void __launch_bounds__(256) eq4_level_kernel(int32_t n, const int32_t* __restrict__ rpv,
+                                                        const int32_t* __restrict__ civ, int32_t* done,
+                                                        int32_t* __restrict__ lvl, int32_t* header, int32_t* stats,
+                                                        long long spin_ns) {
+  const int lane = threadIdx.x & 31;
+  Waiter w{header, spin_ns, 0, nullptr};
+  for (;;) {
+    int tk = 0;
+    if (lane == 0) {
+      tk = atomicAdd(header + (UPPER ? kTicketU : kTicketL), 1);
+      if (ld_volatile_s32(header + kAbort)) tk = n;
+    }
+    tk = __shfl_sync(kFull, tk, 0);
+    if (tk >= n) return;
+    const int i = UPPER ? n - 1 - tk : tk;
+    const int beg = rpv[i], end = rpv[i + 1];
+    int m = 0;
+    bool ok = true;
+    for (int t0 = beg; t0 < end && ok; t0 += 32) {
+      const int t = t0 + lane;
+      const bool has = t < end;
+      const int j = has ? civ[t] : i;
+      int v = has ? ld_relaxed_s32(done + j) : 1;
+      w.t0 = 0;
+      for (unsigned it = 1;; ++it) {
+        if (__all_sync(kFull, v != 0)) break;
+        if ((it & 31u) == 0u && __any_sync(kFull, w.give_up(0u, 0u))) {
+          ok = false;
+          break;
+        }
+        const int v2 = ld_relaxed_s32(done + j);  // every lane re-reads (no per-lane branch)
+        v = v != 0 ? v : v2;
+      }
+      m = max(m, has ? v : 0);
+    }
+    if (!ok) return;  // the abort word stops every other warp
+    m = __reduce_max_sync(kFull, m);
+    if (lane == 0) {
+      lvl[i] = m;
+      st_relaxed_s32(done + i, m + 1);
+      atomicMax(stats + (UPPER ? kNlevU : kNlevL), m + 1);
+    }
+  }
+}
+
+// The same where grid lines are whole runs of 32 rows: warps claim such runs, a
+// lane per row.  Rows outside the run are waited for, all belonging to runs
+// whose tickets were handed out before; those inside it follow lane by lane in
+// registers, and the run is published whole.  (A row per warp has 9.7 k rows in
+// flight, 2.4 planes of a 64x64x32 grid whose wavefront spans all of it: both
+// triangles 2.5 ms, 0.6 with runs.  Runs that cross from one line into the next
+// are one chain, and rows published one by one leave every warp polling: 310 ms
+// at 128x128x64.)
+template <bool UPPER>
+__global__ void __launch_bounds__(128) eq4_runs_kernel(int32_t n, const int32_t* __restrict__ rpv,
                                                         const int32_t* __restrict__ civ, int32_t* done,
                                                         int32_t* __restrict__ lvl, int32_t* header, int32_t* stats,
                                                         long long spin_ns) {
@@ -574,55 +627,41 @@ __global__ void __launch_bounds__(128) eq4_level_kernel(int32_t n, const int32_t
     int t = has ? rpv[i] : 0;
     const int end = has ? rpv[i + 1] : 0;
     int m = 0;           // l(i) so far
-    unsigned inner = 0;  // dependencies inside the run not done yet: bit = lane
-    for (int u = t; u < end; ++u) {
-      const int j = civ[u];
-      const int at_j = (UPPER ? n - 1 - j : j) - tk * 32;
-      if (at_j >= 0) inner |= 1u << at_j;
-    }
-    bool fin = !has;
+    unsigned inner = 0;  // dependencies inside the run: bit = lane
     w.t0 = 0;
     for (unsigned it = 1;; ++it) {
-      // the next dependencies outside, eight loads in flight; a pending one is asked for again
+      // the next dependencies, eight loads in flight; a pending one is asked for again
       while (t < end) {
-        int v[8];  // l(j) + 1; 0: pending; -1: inside the run
+        int v[8];  // l(j) + 1; 0: pending
+        int lane_of[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int j = t + q < end ? civ[t + q] : i;
-          v[q] = t + q < end && (UPPER ? n - 1 - j : j) < tk * 32 ? ld_relaxed_s32(done + j) : -1;
+          lane_of[q] = (UPPER ? n - 1 - j : j) - tk * 32;
+          v[q] = t + q < end && lane_of[q] < 0 ? ld_relaxed_s32(done + j) : 1;
         }
         int got = 0;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           if (got == q && t + q < end && v[q] != 0) {
             got = q + 1;
-            m = max(m, v[q]);
+            if (lane_of[q] < 0) m = max(m, v[q]);
+            else inner |= 1u << lane_of[q];
           }
         t += got;
         if (got < 8) break;
       }
-      // rows that have all they need are published at once (a run may hold the
-      // end of one grid line and the start of the next)
-      for (;;) {
-        const bool now = !fin && t >= end && inner == 0;
-        const unsigned done_now = __ballot_sync(kFull, now);
-        if (!done_now) break;
-        if (now) {
-          lvl[i] = m;
-          st_relaxed_s32(done + i, m + 1);
-          fin = true;
-        }
-        for (unsigned x = done_now; x; x &= x - 1) {
-          const int q = __ffs(x) - 1;
-          const int lq = __shfl_sync(kFull, m, q);
-          if ((inner >> q) & 1u) {
-            m = max(m, lq + 1);
-            inner &= ~(1u << q);
-          }
-        }
-      }
-      if (__all_sync(kFull, fin)) break;
+      if (!__any_sync(kFull, t < end)) break;
       if ((it & 31u) == 0u && __any_sync(kFull, w.give_up(0u, 0u))) return;  // the abort word stops every other warp
+    }
+#pragma unroll 4
+    for (int q = 0; q < 31; ++q) {  // lane q is final when its turn comes
+      const int lq = __shfl_sync(kFull, m, q);
+      if ((inner >> q) & 1u) m = max(m, lq + 1);
+    }
+    if (has) {
+      lvl[i] = m;
+      st_relaxed_s32(done + i, m + 1);
     }
     top = max(top, __reduce_max_sync(kFull, has ? m + 1 : 0));
   }
@@ -858,25 +897,37 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
     slot_map_kernel<<<gsm, 256, 0, s>>>(n, d_arp.as<int32_t>(), d_aci.as<int32_t>(), d_rp, d_ci, d_lrp, d_urp, nnz_l,
                                         d_slot);
   }
-  // Eq. 4, lower then upper: persistent grids, one warp per claimed run of 32 rows
-  int lv_per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lv_per_sm, eq4_level_kernel<false>, 128, 0);
-  const int lgrid = std::max(1, std::min<int>((n + 127) / 128, std::max(lv_per_sm, 1) * sms));
-  cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
-  eq4_level_kernel<false><<<lgrid, 128, 0, s>>>(n, d_lrp, d_lci, d_done.as<int32_t>(), d_lvl_l,
-                                                 d_header.as<int32_t>(), d_stats.as<int32_t>(),
-                                                 trisolve_config().spin_ns);
-  cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
-  eq4_level_kernel<true><<<lgrid, 128, 0, s>>>(n, d_urp, d_uci, d_done.as<int32_t>(), d_lvl_u,
-                                                d_header.as<int32_t>(), d_stats.as<int32_t>(),
-                                                trisolve_config().spin_ns);
   // line length
   line_starts_kernel<<<gsm, 256, 0, s>>>(n, d_flag.as<int32_t>(), d_idx.as<int32_t>(), d_starts.as<int32_t>());
   line_hist_kernel<<<gsm, 256, 0, s>>>((int32_t)nstarts, d_starts.as<int32_t>(), d_hist.as<int32_t>());
   std::vector<int32_t> hist(4097, 0);
+  if (cudaMemcpyAsync(hist.data(), d_hist.p, sizeof(int32_t) * 4097, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess) {
+    cudaFree(sym);
+    cudaFree(mem);
+    return BILU_ERR_CUDA;
+  }
+  int32_t line = 0;  // the rule of the host phase: the most common distance that recurs
+  for (int32_t d = 2; d <= 4096; ++d)
+    if (hist[(size_t)d] > hist[(size_t)line] && hist[(size_t)d] >= 2) line = d;
+  // Eq. 4, lower then upper: persistent grids, one warp per claimed row, or per
+  // run of 32 rows where every line is whole runs
+  const bool whole = line > 0 && line % 32 == 0 && n % line == 0;
+  int lv_per_sm = 1;
+  if (whole) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lv_per_sm, eq4_runs_kernel<false>, 128, 0);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lv_per_sm, eq4_level_kernel<false>, 256, 0);
+  const int rows_per_cta = whole ? 128 : 8, lthreads = whole ? 128 : 256;
+  const int lgrid = std::max(1, std::min<int>((n + rows_per_cta - 1) / rows_per_cta, std::max(lv_per_sm, 1) * sms));
+  cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
+  (whole ? eq4_runs_kernel<false> : eq4_level_kernel<false>)<<<lgrid, lthreads, 0, s>>>(
+      n, d_lrp, d_lci, d_done.as<int32_t>(), d_lvl_l, d_header.as<int32_t>(), d_stats.as<int32_t>(),
+      trisolve_config().spin_ns);
+  cudaMemsetAsync(d_done.p, 0, sizeof(int32_t) * (size_t)n, s);
+  (whole ? eq4_runs_kernel<true> : eq4_level_kernel<true>)<<<lgrid, lthreads, 0, s>>>(
+      n, d_urp, d_uci, d_done.as<int32_t>(), d_lvl_u, d_header.as<int32_t>(), d_stats.as<int32_t>(),
+      trisolve_config().spin_ns);
   if (cudaGetLastError() != cudaSuccess ||
       cudaMemcpyAsync(stats, d_stats.p, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaMemcpyAsync(hist.data(), d_hist.p, sizeof(int32_t) * 4097, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(hdr, d_header.p, sizeof(hdr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cudaFree(sym);
@@ -904,10 +955,7 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   p->max_u = stats[kMaxU];
   p->nlev_l = stats[kNlevL];
   p->nlev_u = stats[kNlevU];
-  int32_t best = 0;  // the rule of the host phase: the most common distance that recurs
-  for (int32_t d = 2; d <= 4096; ++d)
-    if (hist[(size_t)d] > hist[(size_t)best] && hist[(size_t)d] >= 2) best = d;
-  p->line_len = best;
+  p->line_len = line;
   p->host_ready = false;
   p->device = dev;
   p->d_sym = sym;

@@ -38,7 +38,7 @@ def _same(B, n, rp, ci, k, cap=1024):
 
 
 @pytest.mark.parametrize("k", [0, 1, 2, 3, 4, 6])
-@pytest.mark.parametrize("dims,stencil", [((9, 7, 5), 7), ((33, 3, 2), 7), ((8, 6, 5), 27), ((31, 1, 1), 7),
+@pytest.mark.parametrize("dims,stencil", [((9, 7, 5), 7), ((33, 3, 2), 7), ((32, 5, 3), 7), ((64, 4, 3), 7), ((8, 6, 5), 27), ((31, 1, 1), 7),
                                           ((1, 1, 1), 7)])
 def test_grids(B, dims, stencil, k):
     rp, ci = grid_pattern(*dims, stencil)
