@@ -209,29 +209,24 @@ constexpr int kMaxPathLevel = 3;  // longer walks revisit more than a merge does
 constexpr int kPathWarps = 4;
 constexpr int kNever = INT_MAX;
 
-// The checks of bilu_symbolic on the device: row pointers ascending and within
-// nnz before a row's columns are looked at, columns sorted, unique, in range,
-// the diagonal present.
-__global__ void check_kernel(int32_t n, int32_t nnz, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+// The checks of bilu_symbolic's columns on the device (the row pointers are
+// checked on the host): sorted, unique, in range, the diagonal present.
+__global__ void check_kernel(int32_t n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                              int32_t* bad, int32_t* longest) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   int lng = 0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const int beg = rp[i], end = rp[i + 1];
-    bool ok = beg >= 0 && beg <= end && end <= nnz;
-    if (ok) {
-      bool diag = false;
-      int prev = -1;
-      for (int t = beg; t < end && ok; ++t) {
-        const int j = ci[t];
-        ok = j > prev && j < n;
-        diag |= j == (int)i;
-        prev = j;
-      }
-      ok = ok && diag;
-      lng = max(lng, end - beg);
+    bool ok = true, diag = false;
+    int prev = -1;
+    for (int t = beg; t < end && ok; ++t) {
+      const int j = ci[t];
+      ok = j > prev && j < n;
+      diag |= j == (int)i;
+      prev = j;
     }
-    if (!ok) *bad = 1;
+    lng = max(lng, end - beg);
+    if (!ok || !diag) *bad = 1;
   }
   lng = __reduce_max_sync(kFull, lng);
   if ((threadIdx.x & 31) == 0) atomicMax(longest, lng);
@@ -741,6 +736,10 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   if (n == 0) return bilu_symbolic(n, row_ptr, col_idx, k, out);
   if (!row_ptr || (row_ptr[n] > 0 && !col_idx)) return BILU_ERR_ARG;
   if (row_ptr[0] != 0 || row_ptr[n] < n) return BILU_ERR_PATTERN;  // each row holds its diagonal
+  // Ascending row pointers on the host, before row_ptr[n] says how many columns
+  // are read: col_idx holds no more than the row pointers address.
+  for (int32_t i = 0; i < n; ++i)
+    if (row_ptr[i + 1] < row_ptr[i]) return BILU_ERR_PATTERN;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t nnz_a = row_ptr[n];
   const int cap = row_capacity;
@@ -771,7 +770,7 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   cudaMemcpyAsync(d_header.p, hdr, sizeof(hdr), cudaMemcpyHostToDevice, s);
   cudaMemsetAsync(d_stats.p, 0, sizeof(int32_t) * kStatWords, s);
   cudaMemsetAsync(d_hist.p, 0, sizeof(int32_t) * 4097, s);
-  check_kernel<<<gsm, 256, 0, s>>>(n, (int32_t)nnz_a, d_arp.as<int32_t>(), d_aci.as<int32_t>(),
+  check_kernel<<<gsm, 256, 0, s>>>(n, d_arp.as<int32_t>(), d_aci.as<int32_t>(),
                                    d_stats.as<int32_t>() + kBadPattern, d_stats.as<int32_t>() + kLongest);
   if (cudaMemcpyAsync(stats, d_stats.p, sizeof(stats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
