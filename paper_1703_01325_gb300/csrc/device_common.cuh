@@ -10,6 +10,15 @@ namespace bilu {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// The most dynamic shared memory the persistent kernels' CTAs may ask for, beside
+// their static words.  Set as a kernel's limit once per device, never lowered.
+constexpr int kMaxDynamicSmem = 227 * 1024 - 256;
+
+inline int current_device() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
 // "Not yet computed" marker of the sync-free triangular solves: a signalling
 // NaN with a fixed payload.  IEEE arithmetic quiets every signalling NaN it
 // touches, so no computed value carries this bit pattern; a stored value that

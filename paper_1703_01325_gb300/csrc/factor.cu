@@ -23,9 +23,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "device_common.cuh"
+#include "launch_cache.h"
 
 namespace bilu {
 namespace {
@@ -475,9 +475,6 @@ __global__ void __launch_bounds__(256) scale_upper_kernel(int32_t n, const int32
   }
 }
 
-// Dynamic shared memory a CTA may use beside factor_kernel's static word.
-constexpr int kFactorMaxSmem = 227 * 1024 - 256;
-
 int device_sms() {
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -514,17 +511,13 @@ int launch_factor_t(const bilu_pattern* p, int32_t b, TV* f, int32_t* header, in
     // rows of the pattern are at most max_l + 1 + max_u blocks wide
     const int rc = std::min(FactorCap<B>::RC, p->max_l + 1 + p->max_u);
     const size_t smem = factor_smem_bytes<B, TV>(chunk, rc);
-    // the CTAs that fit on an SM, asked for once per shared-memory size: (bytes << 8) | CTAs
-    static std::atomic<unsigned long long> cache{0};
-    unsigned long long have = cache.load(std::memory_order_relaxed);
-    if ((have >> 8) != smem) {
-      cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFactorMaxSmem);
+    static LaunchCache cache;
+    const int per_sm = cache.ctas_per_sm(current_device(), smem, [](size_t bytes) {
+      cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
       int q = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, factor_kernel<B, TV>, FactorCap<B>::W * 32, smem);
-      have = ((unsigned long long)smem << 8) | (unsigned long long)std::max(1, std::min(q, 255));
-      cache.store(have, std::memory_order_relaxed);
-    }
-    const int per_sm = (int)(have & 255);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, factor_kernel<B, TV>, FactorCap<B>::W * 32, bytes);
+      return q;
+    });
     const int grid = std::max(1, std::min(nchunks, per_sm * sms));
     ProfScope ps(BILU_PROF_FACTOR, stream);
     factor_kernel<B, TV><<<grid, FactorCap<B>::W * 32, smem, s>>>(n, chunk, rc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,

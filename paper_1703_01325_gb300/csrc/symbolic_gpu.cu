@@ -42,6 +42,7 @@ namespace bilu {
 namespace {
 
 constexpr int kSymWarps = 4;
+constexpr int kMaxMergeSmem = 227 * 1024;  // symbolic_kernel has no static shared memory
 
 // First index in a[0, len) whose value is >= key (a row of this warp, in
 // shared memory).
@@ -744,7 +745,7 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   const int64_t nnz_a = row_ptr[n];
   const int cap = row_capacity;
   const size_t merge_smem = (size_t)kSymWarps * (4 * (size_t)cap + 32) * sizeof(int);
-  const bool cap_fits = merge_smem <= 227 * 1024;
+  const bool cap_fits = merge_smem <= (size_t)kMaxMergeSmem;
   const long long ntiles = ((long long)n + kScanTile - 1) / kScanTile;
   DevBuf d_arp, d_aci, d_olen, d_done, d_header, d_nl, d_nu, d_flag, d_part, d_stats, d_rp0, d_lrp0, d_urp0, d_idx,
       d_starts, d_hist;
@@ -820,8 +821,8 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
       return BILU_ERR_OOM;
     }
     cudaMemsetAsync(d_done.p, 0, rows, s);
-    cudaFuncSetAttribute(symbolic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)std::max<size_t>(merge_smem, 48 * 1024));
+    // to the most there is: a thread with a smaller row_capacity must not lower it
+    cudaFuncSetAttribute(symbolic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxMergeSmem);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, symbolic_kernel, kSymWarps * 32, merge_smem);
     const int grid = (int)std::max<long long>(1, std::min<long long>((n + kSymWarps - 1) / kSymWarps,

@@ -55,6 +55,7 @@
 #include <algorithm>
 
 #include "device_common.cuh"
+#include "launch_cache.h"
 
 namespace bilu {
 
@@ -408,41 +409,26 @@ __global__ void __launch_bounds__(kTriWarps * 32) tri_solve_kernel(
   }
 }
 
-int sm_count() {
-  static int cached = 0;
-  if (!cached) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev);
-    if (cached <= 0) cached = 1;
-  }
-  return cached;
-}
-
 template <typename TV>
 size_t tri_smem_bytes(int chunk, int b) {
   return align_up16((size_t)chunk * b * sizeof(TV)) + (size_t)chunk * 3 * sizeof(int);
 }
 
-// Persistent grid: as many CTAs as fit on the device at once (cached per
-// shared-memory size; the occupancy query is host work worth skipping per
-// launch).
+// Persistent grid: as many CTAs as fit on the device at once (the occupancy
+// query is host work worth skipping per launch).
 template <int B, bool UPPER, typename TV, int kTriWarps, int GE, typename RT, bool DEEP, bool JOIN>
 int tri_grid(size_t smem, int nchunks) {
-  static size_t last_smem = 0;
-  static int last_per_sm = 1;
-  if (smem != last_smem) {
-    cudaFuncSetAttribute(tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP, JOIN>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
+  static LaunchCache cache;
+  const int fit = cache.ctas_per_sm(current_device(), smem, [](size_t bytes) {
+    auto kernel = tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP, JOIN>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tri_solve_kernel<B, UPPER, TV, kTriWarps, GE, RT, DEEP, JOIN>,
-                                                  kTriWarps * 32, smem);
-    last_per_sm = per_sm < 1 ? 1 : per_sm;
-    last_smem = smem;
-  }
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTriWarps * 32, bytes);
+    return per_sm;
+  });
   const int cap = trisolve_config().ctas_per_sm;
-  const int per_sm = cap > 0 ? std::min(cap, last_per_sm) : last_per_sm;
-  return std::max(1, std::min(nchunks, per_sm * sm_count()));
+  const int per_sm = cap > 0 ? std::min(cap, fit) : fit;
+  return std::max(1, std::min(nchunks, per_sm * device_sm_count()));
 }
 
 // One triangular sweep (the arguments of tri_solve_kernel).
@@ -574,7 +560,7 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
   const TV* L = f;
   const TV* Dinv = f + (size_t)p->nnz_l() * bb;
   const TV* U = Dinv + (size_t)n * bb;
-  const int prep_blocks = (int)std::min<long long>((m + 255) / 256, (long long)sm_count() * 8);
+  const int prep_blocks = (int)std::min<long long>((m + 255) / 256, (long long)device_sm_count() * 8);
   {
     ProfScope ps(BILU_PROF_APPLY_PREP, stream);
     apply_prep_kernel<TV><<<prep_blocks, 256, 0, s>>>(y, xs, m, header, stop);
