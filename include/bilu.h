@@ -129,9 +129,11 @@ int bilu_pattern_upload(bilu_pattern* p, void* stream);
  */
 int bilu_pattern_schedule(bilu_pattern* p, void* stream);
 
-/* Rows per chunk of the current solve and factorization schedules (0 when
- * there is none, e.g. before bilu_pattern_upload).  Either output may be
- * NULL.  Host only. */
+/* Target rows per chunk of the general solve schedule and of the factorization's
+ * (0 when there is none, e.g. before bilu_pattern_upload).  A pattern may hold a
+ * second solve schedule for rows of few blocks (bilu_set_trisolve_chunk(0)):
+ * bilu_apply_info says which one an apply runs on.  Either output may be NULL.
+ * Host only. */
 int bilu_pattern_schedule_info(const bilu_pattern* p, int32_t* solve_rows, int32_t* factor_rows);
 
 /* Frees the handle and its device copy.  NULL is ignored. */

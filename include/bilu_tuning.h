@@ -33,9 +33,17 @@ extern "C" {
 int bilu_set_trisolve_chunk(int32_t rows);
 int32_t bilu_get_trisolve_chunk(void);
 
-/* The target the solves use for pattern p when none is set (bilu_set_trisolve_chunk(0)),
- * for inspection: host pattern, no device work.  Returns -1 for a NULL p. */
+/* The target of pattern p's general solve schedule when none is set
+ * (bilu_set_trisolve_chunk(0)), for inspection: host pattern, no device work.
+ * Returns -1 for a NULL p. */
 int32_t bilu_auto_trisolve_chunk(const bilu_pattern* p);
+
+/* What an apply of p with block size b runs on (f32 != 0: bilu_apply_f32; the
+ * solvers' applies likewise), with the current settings: *rows, the target rows
+ * per chunk of its schedule (0 before bilu_pattern_upload), and *warps, the warps
+ * per CTA of its sweeps.  Either may be NULL.  BILU_ERR_ARG for a NULL p or b
+ * outside 1..8.  Host only. */
+int bilu_apply_info(const bilu_pattern* p, int32_t b, int32_t f32, int32_t* rows, int32_t* warps);
 
 /* Target of consecutive block rows one CTA owns in the sync-free
  * factorization: 0 (the default) picks whole grid lines where a line length L

@@ -78,6 +78,7 @@ SIGNATURES = {
                                        C.c_double, C.c_int32, _vp, C.c_size_t, _vp, C.POINTER(SolveInfo)]),
     "bilu_set_trisolve_chunk": (C.c_int, [C.c_int32]),
     "bilu_get_trisolve_chunk": (C.c_int32, []),
+    "bilu_apply_info": (C.c_int, [_vp, C.c_int32, C.c_int32, _i32p, _i32p]),
     "bilu_set_trisolve_warps": (C.c_int, [C.c_int32]),
     "bilu_set_trisolve_ctas_per_sm": (C.c_int, [C.c_int32]),
     "bilu_auto_trisolve_chunk": (C.c_int32, [C.c_void_p]),

@@ -95,12 +95,20 @@ class Pattern:
         return self
 
     def schedule_info(self) -> dict:
-        """bilu_pattern_schedule_info: rows per chunk of the current solve and
-        factorization schedules."""
+        """bilu_pattern_schedule_info: rows per chunk of the general solve schedule
+        and of the factorization's (apply_info: what an apply runs on)."""
         sr, fr = C.c_int32(), C.c_int32()
         _check(L.load().bilu_pattern_schedule_info(self.handle, C.byref(sr), C.byref(fr)),
                "bilu_pattern_schedule_info")
         return {"solve_rows": sr.value, "factor_rows": fr.value}
+
+    def apply_info(self, b: int, f32: bool = False) -> dict:
+        """bilu_apply_info: target rows per chunk of the schedule an apply with
+        block size b runs on (0 before upload), and the warps per CTA of its
+        sweeps."""
+        rows, warps = C.c_int32(), C.c_int32()
+        _check(L.load().bilu_apply_info(self.handle, b, int(f32), C.byref(rows), C.byref(warps)), "bilu_apply_info")
+        return {"rows": rows.value, "warps": warps.value}
 
     def schedule(self, rows: int) -> dict:
         """The sync-free solve schedule for a target of `rows` rows per chunk

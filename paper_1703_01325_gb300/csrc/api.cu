@@ -500,6 +500,14 @@ extern "C" int32_t bilu_auto_factor_chunk(const bilu_pattern* p) {
   return p ? auto_factor_chunk_target(p) : -1;
 }
 
+extern "C" int bilu_apply_info(const bilu_pattern* p, int32_t b, int32_t f32, int32_t* rows, int32_t* warps) {
+  if (!p || !valid_b(b)) return BILU_ERR_ARG;
+  const bilu_chunk_schedule& s = apply_schedule(p, b, f32 != 0);
+  if (rows) *rows = s.d_mem ? s.chunk : 0;
+  if (warps) *warps = apply_warps(p, b);
+  return BILU_OK;
+}
+
 extern "C" int bilu_set_trisolve_warps(int32_t warps) {
   if (warps != 4 && warps != 8 && warps != 16) return BILU_ERR_ARG;
   trisolve_config().warps = warps;

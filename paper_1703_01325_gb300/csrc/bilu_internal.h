@@ -124,6 +124,9 @@ int32_t solve_chunk_target(const bilu_pattern* p);
 int32_t auto_solve_chunk_target(const bilu_pattern* p);  // the rule alone
 int32_t pair_chunk_target(const bilu_pattern* p);
 bool pair_chunks_fit(const bilu_pattern* p);  // of the built schedule
+// What an apply runs on: the schedule, and the warps per CTA of its sweeps.
+const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32);
+int apply_warps(const bilu_pattern* p, int32_t b);
 int32_t factor_chunk_target(const bilu_pattern* p);
 int32_t auto_factor_chunk_target(const bilu_pattern* p);  // the rule alone
 

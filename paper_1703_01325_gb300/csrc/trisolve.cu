@@ -117,6 +117,22 @@ bool pair_chunks_fit(const bilu_pattern* p) {
   return p->n <= 2.1 * p->line_len * p->pair.nchunks;
 }
 
+const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32) {
+  const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
+  const bool lines = !f32 || p->line_len <= kPairLine;
+  return one_pass && lines && p->pair.d_mem && trisolve_config().warps == 4 ? p->pair : p->solve;
+}
+
+// Rows of many passes: eight warps per CTA, so that a level's rows have been
+// fetched when their turn comes (apply, ms, 4 / 8 warps: 27-point ILU(2) b = 2
+// 128x128x40 6.19 / 4.87, b = 3 80x80x40 6.09 / 5.88, FP32 5.06 / 4.59).  Rows
+// of fewer blocks or passes are not faster (27-point ILU(1) b = 3 2.42 / 2.45;
+// 27-point ILU(2) b = 1, two passes, 1.81 / 1.86).
+int apply_warps(const bilu_pattern* p, int32_t b) {
+  const int set = trisolve_config().warps, widest = std::max(p->max_l, p->max_u);
+  return set == 4 && widest >= 40 && widest > 3 * groups_for(b) ? 8 : set;
+}
+
 int32_t solve_chunk_target(const bilu_pattern* p) {
   const int c = trisolve_config().chunk;
   return c > 0 ? c : auto_solve_chunk_target(p);
@@ -545,9 +561,7 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
   cudaStream_t s = (cudaStream_t)stream;
   const TrisolveConfig& cfg = trisolve_config();
   if (p->solve.chunk <= 0 || !p->solve.upper || !p->solve.d_mem) return (int)cudaErrorInvalidValue;
-  const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
-  const bool lines = sizeof(TV) == 8 || p->line_len <= kPairLine;
-  const bilu_chunk_schedule& sch = one_pass && lines && p->pair.d_mem && cfg.warps == 4 ? p->pair : p->solve;
+  const bilu_chunk_schedule& sch = apply_schedule(p, b, sizeof(TV) == 4);
   int32_t* header = reinterpret_cast<int32_t*>(work);
   const long long m = (long long)n * b;
   // The workspace's vector region holds n*b doubles: y (FP64), or y and the
@@ -565,13 +579,7 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
     ProfScope ps(BILU_PROF_APPLY_PREP, stream);
     apply_prep_kernel<TV><<<prep_blocks, 256, 0, s>>>(y, xs, m, header, stop);
   }
-  // Rows of many passes: eight warps per CTA, so that a level's rows have been
-  // fetched when their turn comes (apply, ms, 4 / 8 warps: 27-point ILU(2) b = 2
-  // 128x128x40 6.19 / 4.87, b = 3 80x80x40 6.09 / 5.88, FP32 5.06 / 4.59).  Rows
-  // of fewer blocks or passes are not faster (27-point ILU(1) b = 3 2.42 / 2.45;
-  // 27-point ILU(2) b = 1, two passes, 1.81 / 1.86).
-  const int widest = std::max(p->max_l, p->max_u);
-  const int warps = cfg.warps == 4 && widest >= 40 && widest > 3 * groups_for(b) ? 8 : cfg.warps;
+  const int warps = apply_warps(p, b);
   BILU_DISPATCH_B(b, {
     if (warps == 16)
       launch_solves<B, TV, 16>(p, sch, L, Dinv, U, r, y, xs, header, cfg, stop, stream);

@@ -1,0 +1,51 @@
+"""bilu_apply_info names the schedule and the warps an apply runs on: the general
+solve schedule, or the second one that rows of one pass run on."""
+from __future__ import annotations
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_1703_01325_gb300.bilu as B  # noqa: E402
+from paper_1703_01325_gb300.reservoir import grid_pattern, reservoir_system  # noqa: E402
+
+
+def test_arguments_and_no_schedule(libbilu):
+    P = B.bilu_symbolic(120, *grid_pattern(6, 5, 4, 7), 1)
+    assert P.apply_info(3)["rows"] == 0 and P.apply_info(3, f32=True)["rows"] == 0
+    for b in (0, 9):
+        with pytest.raises(B.BiluError):
+            P.apply_info(b)
+    assert libbilu.bilu_apply_info(None, 3, 0, None, None) != 0
+    assert libbilu.bilu_apply_info(P.handle, 3, 0, None, None) == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dims,b,k,f64,f32", [
+    ((30, 30, 30), 3, 1, 60, 60),    # one pass: two lines
+    ((30, 30, 30), 5, 0, 60, 60),
+    ((30, 30, 30), 5, 1, 32, 32),    # two passes over four groups: the general schedule
+    ((30, 30, 30), 3, 2, None, None),  # rows of more than eight blocks: no second schedule
+    ((70, 30, 10), 3, 1, 140, 32),   # lines above 64 rows: FP64 only
+    ((70, 30, 10), 3, 0, 32, 32),    # and not for rows of four blocks and fewer
+])
+def test_which_schedule(libbilu, dims, b, k, f64, f32):
+    """... and both schedules give the same bits."""
+    torch.cuda.set_device(0)
+    S = reservoir_system(*dims, b, sigma=1.0, accum=0.01, seed=2)
+    vals, rhs = torch.from_numpy(S.vals.reshape(-1)).cuda(), torch.from_numpy(S.rhs).cuda()
+    P = B.bilu_symbolic_gpu(S.n, S.row_ptr, S.col_idx, k).upload()
+    general = P.schedule_info()["solve_rows"]
+    assert general == B.bilu_auto_trisolve_chunk(P)
+    assert [P.apply_info(b)["rows"], P.apply_info(b, f32=True)["rows"]] == [f64 or general, f32 or general]
+    F, _ = B.bilu_factor(P, b, vals)
+    F32 = B.bilu_convert_f32(F)
+    x, x32 = B.bilu_apply(P, b, F, rhs), B.bilu_apply_f32(P, b, F32, rhs)
+    old = B.bilu_get_trisolve_chunk()
+    try:
+        B.bilu_set_trisolve_chunk(general)
+        P.reschedule()
+    finally:
+        B.bilu_set_trisolve_chunk(old)
+    assert P.apply_info(b)["rows"] == P.apply_info(b, f32=True)["rows"] == general
+    assert torch.equal(B.bilu_apply(P, b, F, rhs), x) and torch.equal(B.bilu_apply_f32(P, b, F32, rhs), x32)
