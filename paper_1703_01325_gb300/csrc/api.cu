@@ -509,7 +509,7 @@ extern "C" int bilu_apply_info(const bilu_pattern* p, int32_t b, int32_t f32, in
 }
 
 extern "C" int bilu_set_trisolve_warps(int32_t warps) {
-  if (warps != 4 && warps != 8 && warps != 16) return BILU_ERR_ARG;
+  if (warps != 0 && warps != 4 && warps != 8 && warps != 16) return BILU_ERR_ARG;
   trisolve_config().warps = warps;
   return BILU_OK;
 }

@@ -107,7 +107,7 @@ constexpr long long kDefaultSpinNs = 2000000000LL;  // 2 s
 // Tunables of the sync-free triangular solves (see trisolve.cu).
 struct TrisolveConfig {
   int chunk = 0;           // target rows per CTA of the solves (0: by size)
-  int warps = 4;           // warps per CTA of the solves (4, 8 or 16)
+  int warps = 0;           // warps per CTA of the solves (4, 8 or 16; 0: apply_warps' rule)
   int ctas_per_sm = 0;     // resident CTAs per SM of the solves (0: as many as fit)
   int factor_chunk = 0;    // target rows per CTA of the factorization (0: by size)
   long long spin_ns = kDefaultSpinNs;

@@ -120,7 +120,7 @@ bool pair_chunks_fit(const bilu_pattern* p) {
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32) {
   const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
   const bool lines = !f32 || p->line_len <= kPairLine;
-  return one_pass && lines && p->pair.d_mem && trisolve_config().warps == 4 ? p->pair : p->solve;
+  return one_pass && lines && p->pair.d_mem && trisolve_config().warps <= 4 ? p->pair : p->solve;
 }
 
 // Rows of many passes: eight warps per CTA, so that a level's rows have been
@@ -130,7 +130,7 @@ const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool
 // 27-point ILU(2) b = 1, two passes, 1.81 / 1.86).
 int apply_warps(const bilu_pattern* p, int32_t b) {
   const int set = trisolve_config().warps, widest = std::max(p->max_l, p->max_u);
-  return set == 4 && widest >= 40 && widest > 3 * groups_for(b) ? 8 : set;
+  return set > 0 ? set : widest >= 40 && widest > 3 * groups_for(b) ? 8 : 4;
 }
 
 int32_t solve_chunk_target(const bilu_pattern* p) {

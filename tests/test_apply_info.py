@@ -20,6 +20,20 @@ def test_arguments_and_no_schedule(libbilu):
     assert libbilu.bilu_apply_info(P.handle, 3, 0, None, None) == 0
 
 
+def test_warps_that_are_set_are_used(libbilu):
+    """A 27-point ILU(2) row has up to 60 blocks a side: eight warps unless 4 is set."""
+    rp, ci = grid_pattern(9, 8, 7, 27)
+    P = B.bilu_symbolic(504, rp, ci, 2)
+    try:
+        B.bilu_set_trisolve_warps(0)
+        assert [P.apply_info(b)["warps"] for b in (1, 2, 3, 8)] == [4, 8, 8, 8]
+        for w in (4, 8, 16):
+            B.bilu_set_trisolve_warps(w)
+            assert [P.apply_info(b)["warps"] for b in (1, 3, 8)] == [w] * 3
+    finally:
+        B.bilu_set_trisolve_warps(0)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("dims,b,k,f64,f32", [
     ((30, 30, 30), 3, 1, 60, 60),    # one pass: two lines
@@ -32,6 +46,7 @@ def test_arguments_and_no_schedule(libbilu):
 def test_which_schedule(libbilu, dims, b, k, f64, f32):
     """... and both schedules give the same bits."""
     torch.cuda.set_device(0)
+    B.bilu_set_trisolve_warps(0)
     S = reservoir_system(*dims, b, sigma=1.0, accum=0.01, seed=2)
     vals, rhs = torch.from_numpy(S.vals.reshape(-1)).cuda(), torch.from_numpy(S.rhs).cuda()
     P = B.bilu_symbolic_gpu(S.n, S.row_ptr, S.col_idx, k).upload()
