@@ -112,6 +112,11 @@ int bilu_set_check_every(int32_t iters);
  * and the call reports BILU_ERR_TIMEOUT.  -1 (the default) disables it. */
 int bilu_test_withhold_row(int32_t row);
 
+/* Test hook: device allocations of at least `bytes` bytes that the schedules'
+ * set-up asks for fail after the first `skip` of them, as if memory had run out.
+ * 0 bytes (the default) disables it.  BILU_ERR_ARG for a negative argument. */
+int bilu_test_fail_alloc(int64_t bytes, int32_t skip);
+
 /* Kernel classes for bilu_profile_read. */
 enum bilu_prof_kernel {
   BILU_PROF_SPMV = 0,         /* bsr_spmv kernel */

@@ -87,6 +87,7 @@ SIGNATURES = {
     "bilu_get_factor_chunk": (C.c_int32, []),
     "bilu_set_spin_limit_ns": (C.c_int, [C.c_int64]),
     "bilu_set_check_every": (C.c_int, [C.c_int32]),
+    "bilu_test_fail_alloc": (C.c_int, [C.c_int64, C.c_int32]),
     "bilu_test_withhold_row": (C.c_int, [C.c_int32]),
     "bilu_profile_enable": (C.c_int, [C.c_int32]),
     "bilu_profile_read": (C.c_int, [C.c_int32, C.POINTER(C.c_int64), C.POINTER(C.c_double)]),

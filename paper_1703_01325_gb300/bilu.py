@@ -474,6 +474,10 @@ def bilu_set_check_every(iters: int):
     _check(L.load().bilu_set_check_every(iters), "bilu_set_check_every")
 
 
+def bilu_test_fail_alloc(nbytes: int, skip: int = 0):
+    _check(L.load().bilu_test_fail_alloc(nbytes, skip), "bilu_test_fail_alloc")
+
+
 def bilu_test_withhold_row(row: int):
     _check(L.load().bilu_test_withhold_row(row), "bilu_test_withhold_row")
 

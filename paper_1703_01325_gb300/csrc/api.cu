@@ -537,6 +537,13 @@ extern "C" int bilu_test_withhold_row(int32_t row) {
   return BILU_OK;
 }
 
+extern "C" int bilu_test_fail_alloc(int64_t bytes, int32_t skip) {
+  if (bytes < 0 || skip < 0) return BILU_ERR_ARG;
+  trisolve_config().fail_bytes = bytes;
+  trisolve_config().fail_skip = skip;
+  return BILU_OK;
+}
+
 extern "C" int bilu_schedule_export(const bilu_pattern* p, int32_t rows, int32_t* nchunks, int32_t* bounds,
                                     int32_t* ord_lower, int32_t* ord_upper, int32_t* tick_lower,
                                     int32_t* tick_upper) {

@@ -107,6 +107,8 @@ constexpr long long kDefaultSpinNs = 2000000000LL;  // 2 s
 // Tunables of the sync-free triangular solves (see trisolve.cu).
 struct TrisolveConfig {
   int chunk = 0;           // target rows per CTA of the solves (0: by size)
+  int64_t fail_bytes = 0;  // bilu_test_fail_alloc
+  int32_t fail_skip = 0;
   int warps = 0;           // warps per CTA of the solves (4, 8 or 16; 0: apply_warps' rule)
   int ctas_per_sm = 0;     // resident CTAs per SM of the solves (0: as many as fit)
   int factor_chunk = 0;    // target rows per CTA of the factorization (0: by size)
@@ -196,6 +198,7 @@ void ticket_order_lists(int32_t nchunks, const std::vector<int32_t>& prio, const
 struct ScheduleInputs {
   std::vector<int32_t> gapl, gapu;
   int32_t *d_lvl_l = nullptr, *d_lvl_u = nullptr;
+  bool many_preds = false;  // a chunk had more predecessors than the gathered lists hold
   ScheduleInputs() = default;
   ScheduleInputs(const ScheduleInputs&) = delete;
   ~ScheduleInputs();

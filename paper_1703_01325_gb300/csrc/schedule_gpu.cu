@@ -145,9 +145,16 @@ __global__ void chunk_edges_kernel(int32_t nchunks, const int32_t* __restrict__ 
 // The same for chunks with at most kMaxPreds distinct predecessors, in one
 // pass: a CTA per chunk gathers them in a set in shared memory (4 kMaxPreds
 // slots) and writes them, in any order, at preds[c * kMaxPreds].  A chunk with
-// more sets *over.  (A warp walking the chunk's rows, then sorting and
-// uniting the lists, took 0.7 ms a triangle on a 64x64x32 grid; this, 0.1 ms.)
+// more sets *over, and every CTA leaves once it sees that.  (A warp walking the
+// chunk's rows, then sorting and uniting the lists, took 0.7 ms a triangle on a
+// 64x64x32 grid; this, 0.1 ms.  20,000 rows of 30 columns anywhere: upload 2.57 ms
+// with the lists alone, 4.43 when every chunk of every schedule was gathered before
+// *over was looked at, 2.55 now, with one look per pattern.)
 constexpr int kMaxPreds = 64;
+
+// Whether the gathered lists are worth their memory, kMaxPreds words a chunk: for
+// chunks of eight rows and more on average (at most 32 bytes a row).
+bool gathers_preds(int32_t n, int32_t nchunks) { return (long long)nchunks * 8 <= n; }
 
 template <bool UPPER>
 __global__ void __launch_bounds__(128) chunk_preds_kernel(int32_t nchunks, const int32_t* __restrict__ bnd,
@@ -157,14 +164,16 @@ __global__ void __launch_bounds__(128) chunk_preds_kernel(int32_t nchunks, const
                                                           int32_t* __restrict__ count, int32_t* __restrict__ preds,
                                                           int32_t* __restrict__ over) {
   __shared__ int set[4 * kMaxPreds];
-  __shared__ int s_n, s_prio;
+  __shared__ int s_n, s_prio, s_over;
   for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    if (threadIdx.x == 0) s_over = ld_volatile_s32(over);
     for (int q = threadIdx.x; q < 4 * kMaxPreds; q += blockDim.x) set[q] = -1;
     if (threadIdx.x == 0) {
       s_n = 0;
       s_prio = INT_MAX;
     }
     __syncthreads();
+    if (s_over) return;  // read by the whole CTA between two barriers
     const int lc = UPPER ? nchunks - 1 - c : c;
     const int lo = bnd[lc], hi = bnd[lc + 1];
     int pm = INT_MAX;
@@ -174,6 +183,7 @@ __global__ void __launch_bounds__(128) chunk_preds_kernel(int32_t nchunks, const
       for (int t = rpv[i]; t < rpv[i + 1]; ++t) {
         const int j = civ[t];
         if ((j >= lo && j < hi) || (j >= a && j < z)) continue;
+        if (*reinterpret_cast<volatile int*>(&s_n) > kMaxPreds) break;
         const int lj = chunk_of_row(bnd, nchunks, j);
         a = bnd[lj];
         z = bnd[lj + 1];
@@ -239,6 +249,13 @@ __global__ void pack_kernel(int32_t nchunks, const int64_t* __restrict__ off, co
     for (long long t = lane; t < ucount[c]; t += 32) packed[uoff[c] + t] = uniq[off[c] + t];
 }
 
+// cudaMalloc of the schedules' set-up, with the test hook's failures.
+cudaError_t schedule_malloc(void** p, size_t bytes) {
+  TrisolveConfig& cfg = trisolve_config();
+  if (cfg.fail_bytes > 0 && bytes >= (size_t)cfg.fail_bytes && cfg.fail_skip-- <= 0) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 // Device scratch freed on every return path.
 struct Scratch {
   std::vector<void*> bufs;
@@ -248,7 +265,7 @@ struct Scratch {
   template <typename T>
   T* get(size_t count) {
     void* p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(count * sizeof(T), 16)) != cudaSuccess) {
+    if (schedule_malloc(&p, std::max<size_t>(count * sizeof(T), 16)) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
@@ -268,36 +285,39 @@ int device_sms() {
 // the device, list scheduling on the host (work per chunk, not per entry).
 template <bool UPPER>
 int ticket_order_device(const bilu_pattern* p, const bilu_chunk_schedule* s, const int32_t* d_bnd,
-                        const int32_t* lvl, std::vector<int32_t>& tick) {
+                        const int32_t* lvl, ScheduleInputs* in, std::vector<int32_t>& tick) {
   const int32_t nchunks = s->nchunks;
   const int32_t* rpv = UPPER ? p->d_urp : p->d_lrp;
   const int32_t* civ = UPPER ? p->d_uci : p->d_lci;
   const int grid = device_sms() * 8;
-  {
+  if (!in->many_preds && gathers_preds(p->n, nchunks)) {
     Scratch few;
     const size_t nc = (size_t)nchunks;
     int32_t* d_all = few.get<int32_t>(1 + 2 * nc + nc * kMaxPreds);  // over | prio | count | preds
-    if (!d_all) return BILU_ERR_OOM;
-    cudaMemsetAsync(d_all, 0, sizeof(int32_t));
-    chunk_preds_kernel<UPPER><<<std::min(nchunks, grid), 128>>>(nchunks, d_bnd, rpv, civ, lvl, d_all + 1,
-                                                                d_all + 1 + nc, d_all + 1 + 2 * nc, d_all);
-    std::vector<int32_t> all(1 + 2 * nc + nc * kMaxPreds);
-    if (cudaMemcpy(all.data(), d_all, sizeof(int32_t) * all.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
-      return BILU_ERR_CUDA;
-    if (!all[0]) {
-      const std::vector<int32_t> prio(all.begin() + 1, all.begin() + 1 + nchunks);
-      std::vector<int32_t> pred;
-      std::vector<int64_t> pred_ptr(nc + 1, 0);
-      for (size_t c = 0; c < nc; ++c) {
-        const int32_t* const from = all.data() + 1 + 2 * nc + c * kMaxPreds;
-        pred.insert(pred.end(), from, from + all[1 + nc + c]);
-        pred_ptr[c + 1] = (int64_t)pred.size();
+    if (d_all) {
+      cudaMemsetAsync(d_all, 0, sizeof(int32_t));
+      chunk_preds_kernel<UPPER><<<std::min(nchunks, grid), 128>>>(nchunks, d_bnd, rpv, civ, lvl, d_all + 1,
+                                                                  d_all + 1 + nc, d_all + 1 + 2 * nc, d_all);
+      std::vector<int32_t> all(1 + 2 * nc + nc * kMaxPreds);
+      if (cudaMemcpy(all.data(), d_all, sizeof(int32_t) * all.size(), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return BILU_ERR_CUDA;
+      if (!all[0]) {
+        const std::vector<int32_t> prio(all.begin() + 1, all.begin() + 1 + nchunks);
+        std::vector<int32_t> pred;
+        std::vector<int64_t> pred_ptr(nc + 1, 0);
+        for (size_t c = 0; c < nc; ++c) {
+          const int32_t* const from = all.data() + 1 + 2 * nc + c * kMaxPreds;
+          pred.insert(pred.end(), from, from + all[1 + nc + c]);
+          pred_ptr[c + 1] = (int64_t)pred.size();
+        }
+        ticket_order_lists(nchunks, prio, pred_ptr, pred, tick);
+        return BILU_OK;
       }
-      ticket_order_lists(nchunks, prio, pred_ptr, pred, tick);
-      return BILU_OK;
+      in->many_preds = true;
     }
   }
-  // many predecessors (irregular patterns): lists of any length
+  // many predecessors (irregular patterns), short chunks, or no memory for the
+  // gathered lists: lists of any length
   Scratch sc;
   int32_t* d_prio = sc.get<int32_t>((size_t)nchunks);
   int64_t* d_count = sc.get<int64_t>((size_t)nchunks + 1);
@@ -355,7 +375,7 @@ bool ScheduleInputs::levels(const bilu_pattern* p) {
   if (d_lvl_l || p->d_lvl_l) return true;
   const size_t n = (size_t)p->n;
   void* m = nullptr;
-  if (cudaMalloc(&m, 2 * n * sizeof(int32_t)) != cudaSuccess) {
+  if (schedule_malloc(&m, 2 * n * sizeof(int32_t)) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -402,7 +422,7 @@ int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bil
     const size_t bd = align256(sizeof(int32_t) * ((size_t)nchunks + 1));
     const int parts = upper ? 2 : 1;
     void* mem = nullptr;
-    if (cudaMalloc(&mem, bd + parts * (one + tk)) != cudaSuccess) {
+    if (schedule_malloc(&mem, bd + parts * (one + tk)) != cudaSuccess) {
       cudaGetLastError();
       return BILU_ERR_OOM;
     }
@@ -420,9 +440,9 @@ int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bil
     chunk_order_kernel<false><<<ogrid, kOrderWarps * 32>>>(nchunks, s->d_bnd, p->d_lrp, p->d_lci, s->d_ord_l);
     if (upper)
       chunk_order_kernel<true><<<ogrid, kOrderWarps * 32>>>(nchunks, s->d_bnd, p->d_urp, p->d_uci, s->d_ord_u);
-    int st = ticket_order_device<false>(p, s, s->d_bnd, in->d_lvl_l ? in->d_lvl_l : p->d_lvl_l, s->tick_l);
+    int st = ticket_order_device<false>(p, s, s->d_bnd, in->d_lvl_l ? in->d_lvl_l : p->d_lvl_l, in, s->tick_l);
     if (st == BILU_OK && upper)
-      st = ticket_order_device<true>(p, s, s->d_bnd, in->d_lvl_u ? in->d_lvl_u : p->d_lvl_u, s->tick_u);
+      st = ticket_order_device<true>(p, s, s->d_bnd, in->d_lvl_u ? in->d_lvl_u : p->d_lvl_u, in, s->tick_u);
     if (st == BILU_OK) {
       cudaMemcpy(s->d_tick_l, s->tick_l.data(), sizeof(int32_t) * (size_t)nchunks, cudaMemcpyHostToDevice);
       if (upper)
