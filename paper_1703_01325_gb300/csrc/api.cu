@@ -6,6 +6,7 @@
 
 #include <cstring>
 #include <new>
+#include <utility>
 
 #include "../../include/bilu_tuning.h"
 #include "bilu_internal.h"
@@ -24,13 +25,23 @@ int solve_schedule(const bilu_pattern* p) {
 }
 int factor_schedule(const bilu_pattern* p) { return (p->n == 0 || p->fact.d_mem) ? BILU_OK : BILU_ERR_STATE; }
 
+// All new before any old one goes: on failure the old ones stay.  The second solve
+// schedule is one the applies can do without, so a failure there only leaves it out.
 int build_schedules(bilu_pattern* p) {
   ScheduleInputs in;
-  if (make_schedule(p, &p->solve, solve_chunk_target(p), true, &in) != 0) return BILU_ERR_OOM;
-  const int32_t pair = pair_chunk_target(p);
-  if (pair > 0 && make_schedule(p, &p->pair, pair, true, &in) != 0) return BILU_ERR_OOM;
-  if (pair == 0 || !pair_chunks_fit(p)) free_schedule(&p->pair);
-  if (!p->is_transpose && make_schedule(p, &p->fact, factor_chunk_target(p), false, &in) != 0) return BILU_ERR_OOM;
+  bilu_chunk_schedule solve, pair, fact;
+  int st = make_schedule(p, &solve, solve_chunk_target(p), true, &in);
+  if (st == BILU_OK && !p->is_transpose) st = make_schedule(p, &fact, factor_chunk_target(p), false, &in);
+  if (st != BILU_OK) {
+    free_schedule(&solve);
+    return st;
+  }
+  const int32_t target = pair_chunk_target(p);
+  if (target > 0 && make_schedule(p, &pair, target, true, &in, pair_least_chunks(p)) != BILU_OK) cudaGetLastError();
+  std::swap(p->solve, solve);
+  std::swap(p->pair, pair);
+  std::swap(p->fact, fact);
+  for (bilu_chunk_schedule* old : {&solve, &pair, &fact}) free_schedule(old);
   return BILU_OK;
 }
 

@@ -125,7 +125,7 @@ TrisolveConfig& trisolve_config();
 int32_t solve_chunk_target(const bilu_pattern* p);
 int32_t auto_solve_chunk_target(const bilu_pattern* p);  // the rule alone
 int32_t pair_chunk_target(const bilu_pattern* p);
-bool pair_chunks_fit(const bilu_pattern* p);  // of the built schedule
+int32_t pair_least_chunks(const bilu_pattern* p);  // fewer would hold more than two lines each
 // What an apply runs on: the schedule, and the warps per CTA of its sweeps.
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32);
 int apply_warps(const bilu_pattern* p, int32_t b);
@@ -173,11 +173,13 @@ int launch_factor_f32(const bilu_pattern* p, int32_t b, float* f, int32_t* heade
 int launch_scale_upper_f32(const bilu_pattern* p, int32_t b, float* f, void* stream);
 
 size_t apply_workspace_bytes(int32_t n, int32_t b);
-// Builds (host) and uploads schedule *s for `chunk` rows per chunk (the U'
-// part only if `upper`).  Allocates device memory and synchronises; the
-// previous schedule is freed only once the new one is in place.
+// Builds schedule *s (empty) on the device for `chunk` rows per chunk (the U' part
+// only if `upper`); it stays empty, with BILU_OK, where the cuts make fewer than
+// `least` chunks.  Allocates device memory and synchronises.  BILU_ERR_OOM on
+// failure, *s empty.
 struct ScheduleInputs;
-int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in);
+int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in,
+                  int32_t least = 0);
 // Host part (symbolic.cpp).
 void build_schedule(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
 // The parts of a schedule both builders share (symbolic.cpp): chunk cuts from
@@ -205,7 +207,7 @@ struct ScheduleInputs {
   bool levels(const bilu_pattern* p);  // copies them up if need be
 };
 int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s,
-                          ScheduleInputs* in = nullptr);
+                          ScheduleInputs* in = nullptr, int32_t least = 0);
 // Eq. 4 levels, L / U' split and backfill map of a pattern with rp, ci, lev set.
 int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col_idx);
 // Fills the host vectors of a device-built pattern from its device copies

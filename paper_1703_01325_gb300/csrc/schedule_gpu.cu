@@ -386,7 +386,7 @@ bool ScheduleInputs::levels(const bilu_pattern* p) {
 }
 
 int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bilu_chunk_schedule* s,
-                          ScheduleInputs* in) {
+                          ScheduleInputs* in, int32_t least) {
   const int32_t n = p->n;
   s->chunk = target;
   s->upper = upper;
@@ -417,6 +417,7 @@ int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bil
     schedule_cuts(n, target, upper, in->gapl, in->gapu, s);
     if (s->max_len > kMaxChunkRows) return BILU_ERR_ARG;
     const int32_t nchunks = s->nchunks;
+    if (nchunks < least) return BILU_OK;
     const size_t one = align256(sizeof(int32_t) * (size_t)n);
     const size_t tk = align256(sizeof(int32_t) * (size_t)nchunks);
     const size_t bd = align256(sizeof(int32_t) * ((size_t)nchunks + 1));

@@ -53,6 +53,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "device_common.cuh"
 #include "launch_cache.h"
@@ -100,7 +101,7 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // 61x47x33 ILU(0) b = 5 310 / 293, 150x30x20 ILU(1) b = 4 465 / 394); rows of
 // two passes are not (b = 5 ILU(1) 883 / 967, b = 6 874 / 937), nor grids whose
 // few lines per plane leave chunks of three (100x9x60 ILU(0) b = 8: 379 / 405;
-// pair_chunks_fit).  Two long lines hold a chunk too long where a row is quick:
+// pair_least_chunks).  Two long lines hold a chunk too long where a row is quick:
 // beyond kPairLine only FP64 rows of more than four blocks (FP32 105x21x9 ILU(0)
 // b = 4: 142 / 164; FP64 100x9x60 ILU(1) b = 3: 521 / 472).
 constexpr int kPairLine = 64;
@@ -113,9 +114,7 @@ int32_t pair_chunk_target(const bilu_pattern* p) {
   return 2 * p->line_len;
 }
 
-bool pair_chunks_fit(const bilu_pattern* p) {
-  return p->n <= 2.1 * p->line_len * p->pair.nchunks;
-}
+int32_t pair_least_chunks(const bilu_pattern* p) { return (int32_t)std::ceil(p->n / (2.1 * p->line_len)); }
 
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32) {
   const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
@@ -609,14 +608,13 @@ void free_schedule(bilu_chunk_schedule* s) {
   s->chunk = 0;
 }
 
-int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in) {
+int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in,
+                  int32_t least) {
   // on the device also for patterns completed on the host: the same schedule
   // (64x64x32 ILU(1), three schedules of a pattern: 23 ms on the host, 2 here)
-  bilu_chunk_schedule t;
-  if (build_schedule_device(p, chunk, upper, &t, in) != BILU_OK) return (int)cudaErrorMemoryAllocation;
+  if (build_schedule_device(p, chunk, upper, s, in, least) == BILU_OK) return BILU_OK;
   free_schedule(s);
-  *s = std::move(t);
-  return 0;
+  return BILU_ERR_OOM;
 }
 
 size_t apply_workspace_bytes(int32_t n, int32_t b) {

@@ -45,3 +45,47 @@ def test_many_predecessors(n, density, rows):
     """Every chunk depends on more chunks than the gathered lists hold (64); some before 65 rows of work."""
     rp, ci = random_pattern(n, density=density, seed=n + rows)
     _same_schedule(B.bilu_symbolic_gpu(n, rp, ci, 0, row_capacity=1024), B.bilu_symbolic(n, rp, ci, 0), rows)
+
+
+def _apply_of(P):
+    """Status and result of an apply (b = 3) with fixed factors and right-hand side."""
+    g = torch.Generator().manual_seed(1)
+    F = (torch.rand(P.factor_bytes(3) // 8, generator=g, dtype=torch.float64) * 0.01).cuda()
+    return B.bilu_apply(P, 3, F, torch.rand(27000 * 3, generator=g, dtype=torch.float64).cuda()).clone()
+
+
+def test_second_schedule_is_left_out_without_memory(libbilu):
+    """A 30^3 ILU(1) grid: 226 KB the general schedule, 223 KB each of its two gathered lists, 221 KB the second
+    schedule (which fails), 112 KB the factorization's."""
+    P = B.bilu_symbolic_gpu(27000, *grid_pattern(30, 30, 30, 7), 1)
+    B.bilu_test_fail_alloc(215 << 10, 3)
+    P.upload()
+    assert P.schedule_info() == {"solve_rows": 32, "factor_rows": 60} and P.apply_info(3)["rows"] == 32
+    x = _apply_of(P)
+    B.bilu_test_fail_alloc(0)
+    P.reschedule()
+    assert P.apply_info(3)["rows"] == 60
+    assert torch.equal(_apply_of(P), x)
+
+
+def test_failed_reschedule_leaves_all_old_schedules(libbilu):
+    """The factorization's schedule fails (the sixth allocation of 100 KB and more: two of row gaps, the general
+    schedule, its two gathered lists, this): no schedule of the new setting is in place."""
+    from paper_1703_01325_gb300 import _lib as L
+    P = B.bilu_symbolic_gpu(27000, *grid_pattern(30, 30, 30, 7), 1).upload()
+    before = (P.schedule_info(), P.apply_info(3), P.apply_info(6))
+    x = _apply_of(P)
+    try:
+        B.bilu_set_trisolve_chunk(40)
+        B.bilu_test_fail_alloc(100 << 10, 5)
+        with pytest.raises(B.BiluError) as e:
+            P.reschedule()
+        assert e.value.status == L.BILU_ERR_OOM
+        assert (P.schedule_info(), P.apply_info(3), P.apply_info(6)) == before
+        assert torch.equal(_apply_of(P), x)
+        B.bilu_test_fail_alloc(0)
+        P.reschedule()
+        assert P.schedule_info()["solve_rows"] == P.apply_info(3)["rows"] == 40
+        assert torch.equal(_apply_of(P), x)
+    finally:
+        B.bilu_set_trisolve_chunk(0)
