@@ -47,6 +47,7 @@ struct bilu_pattern {
   // their predecessor (grid-line starts in a natural ordering: the line
   // length); 0 if no distance recurs.
   int32_t line_len = 0;
+  int32_t line_starts = 0;  // such rows (n / line_len of them if every line is that long)
   // Backfill gather map: for every factor slot in [L | D | U] the A block that
   // lands there, or -1 for a fill block (Algorithm 5 steps 3-4).  For a
   // transposed pattern (is_transpose): the slot of the source pattern's factor

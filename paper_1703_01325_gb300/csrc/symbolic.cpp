@@ -72,7 +72,7 @@ void finish_pattern(bilu_pattern* p) {
   p->nlev_u = mu + 1;
 
   // Split P' into strictly lower and strictly upper CSR structures.
-  p->max_l = p->max_u = p->line_len = 0;
+  p->max_l = p->max_u = p->line_len = p->line_starts = 0;
   p->lrp.assign((size_t)n + 1, 0);
   p->urp.assign((size_t)n + 1, 0);
   for (int32_t i = 0; i < n; ++i) {
@@ -106,6 +106,7 @@ void finish_pattern(bilu_pattern* p) {
   for (int32_t i = 0; i < n; ++i) {
     const int32_t e = p->lrp[(size_t)i + 1];
     if (e > p->lrp[i] && p->lci[(size_t)e - 1] == i - 1) continue;  // depends on its predecessor
+    ++p->line_starts;
     if (prev >= 0 && i - prev <= 4096) ++hist[(size_t)(i - prev)];
     prev = i;
   }

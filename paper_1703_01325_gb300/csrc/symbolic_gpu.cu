@@ -956,6 +956,7 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   p->nlev_l = stats[kNlevL];
   p->nlev_u = stats[kNlevU];
   p->line_len = line;
+  p->line_starts = (int32_t)nstarts;
   p->host_ready = false;
   p->device = dev;
   p->d_sym = sym;

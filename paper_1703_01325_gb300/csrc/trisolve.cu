@@ -103,12 +103,17 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // few lines per plane leave chunks of three (100x9x60 ILU(0) b = 8: 379 / 405;
 // pair_least_chunks).  Two long lines hold a chunk too long where a row is quick:
 // beyond kPairLine only FP64 rows of more than four blocks (FP32 105x21x9 ILU(0)
-// b = 4: 142 / 164; FP64 100x9x60 ILU(1) b = 3: 521 / 472).
+// b = 4: 142 / 164; FP64 100x9x60 ILU(1) b = 3: 521 / 472).  And only where every
+// line has the same length: where cells are missing, two lines of a chunk are out
+// of step (grids whose lines each lost up to a share of their cells, ILU(1) b = 3,
+// general schedule / two lines: 40x40x20, a fifth 272 / 381, half 266 / 553;
+// 30x30x30, 0.3 283 / 377; 64x64x32, 0.3 470 / 472, 0.6 563 / 536).
 constexpr int kPairLine = 64;
 
 int32_t pair_chunk_target(const bilu_pattern* p) {
   const int widest = std::max(p->max_l, p->max_u);
   if (trisolve_config().chunk > 0 || p->line_len < 16 || p->line_len > 192 || widest > 8 ||
+      (long long)p->line_starts * p->line_len != p->n ||
       (p->line_len > kPairLine && widest <= 4) || auto_solve_chunk_target(p) == 2 * p->line_len)
     return 0;
   return 2 * p->line_len;

@@ -2,6 +2,7 @@
 solve schedule, or the second one that rows of one pass run on."""
 from __future__ import annotations
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -64,3 +65,22 @@ def test_which_schedule(libbilu, dims, b, k, f64, f32):
         B.bilu_set_trisolve_chunk(old)
     assert P.apply_info(b)["rows"] == P.apply_info(b, f32=True)["rows"] == general
     assert torch.equal(B.bilu_apply(P, b, F, rhs), x) and torch.equal(B.bilu_apply_f32(P, b, F32, rhs), x32)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("host", [True, False])
+def test_lines_of_all_lengths_take_the_general_schedule(libbilu, host):
+    """A grid whose lines lost cells at their ends has lines of 20 to 30 rows, most of them of 30."""
+    torch.cuda.set_device(0)
+    B.bilu_set_trisolve_warps(0)
+    rp, ci = grid_pattern(30, 30, 30, 7)
+    rng = np.random.default_rng(4)
+    lost = np.where(rng.random(900) < 0.4, rng.integers(1, 11, 900), 0)
+    keep = np.arange(27000) % 30 < 30 - np.repeat(lost, 30)
+    new, rows = np.cumsum(keep) - 1, np.repeat(np.arange(27000), np.diff(rp))
+    ok = keep[rows] & keep[ci]
+    n = int(keep.sum())
+    rp = np.concatenate([[0], np.cumsum(np.bincount(new[rows[ok]], minlength=n))]).astype(np.int32)
+    ci = new[ci[ok]].astype(np.int32)
+    P = (B.bilu_symbolic(n, rp, ci, 1) if host else B.bilu_symbolic_gpu(n, rp, ci, 1)).upload()
+    assert P.apply_info(3)["rows"] == P.apply_info(3, f32=True)["rows"] == P.schedule_info()["solve_rows"]
