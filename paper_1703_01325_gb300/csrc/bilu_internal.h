@@ -174,7 +174,7 @@ int launch_factor_f32(const bilu_pattern* p, int32_t b, float* f, int32_t* heade
 int launch_scale_upper_f32(const bilu_pattern* p, int32_t b, float* f, void* stream);
 
 size_t apply_workspace_bytes(int32_t n, int32_t b);
-// Builds schedule *s (empty) on the device for `chunk` rows per chunk (the U' part
+// Builds schedule *s (empty) for `chunk` rows per chunk (the U' part
 // only if `upper`); it stays empty, with BILU_OK, where the cuts make fewer than
 // `least` chunks.  Allocates device memory and synchronises.  BILU_ERR_OOM on
 // failure, *s empty.
@@ -182,7 +182,7 @@ struct ScheduleInputs;
 int make_schedule(const bilu_pattern* p, bilu_chunk_schedule* s, int32_t chunk, bool upper, ScheduleInputs* in,
                   int32_t least = 0);
 // Host part (symbolic.cpp).
-void build_schedule(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s);
+void build_schedule(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s, int32_t least = 0);
 // The parts of a schedule both builders share (symbolic.cpp): chunk cuts from
 // the per-row gaps (gapl[r] = r - the last column of L(r), gapu[r] = the first
 // column of U'(r-1) - (r-1), INT32_MAX where there is none), and the claim
@@ -209,6 +209,7 @@ struct ScheduleInputs {
 };
 int build_schedule_device(const bilu_pattern* p, int32_t chunk, bool upper, bilu_chunk_schedule* s,
                           ScheduleInputs* in = nullptr, int32_t least = 0);
+int upload_schedule(int32_t n, bilu_chunk_schedule* s);
 // Eq. 4 levels, L / U' split and backfill map of a pattern with rp, ci, lev set.
 int complete_pattern(bilu_pattern* p, const int32_t* row_ptr, const int32_t* col_idx);
 // Fills the host vectors of a device-built pattern from its device copies

@@ -385,6 +385,33 @@ bool ScheduleInputs::levels(const bilu_pattern* p) {
          cudaMemcpy(d_lvl_u, p->lvl_u.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
+// The device copy of a schedule the host builder made: what the kernels read.
+int upload_schedule(int32_t n, bilu_chunk_schedule* s) {
+  const size_t one = align256(sizeof(int32_t) * (size_t)n);
+  const size_t tk = align256(sizeof(int32_t) * (size_t)s->nchunks);
+  const size_t bd = align256(sizeof(int32_t) * ((size_t)s->nchunks + 1));
+  if (schedule_malloc(&s->d_mem, bd + (s->upper ? 2 : 1) * (one + tk)) != cudaSuccess) {
+    cudaGetLastError();
+    s->d_mem = nullptr;
+    return BILU_ERR_OOM;
+  }
+  char* m = (char*)s->d_mem;
+  bool ok = true;
+  auto put = [&](int32_t*& dst, const std::vector<int32_t>& v, size_t bytes) {
+    dst = (int32_t*)m;
+    m += bytes;
+    ok = ok && cudaMemcpy(dst, v.data(), sizeof(int32_t) * v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  };
+  put(s->d_bnd, s->bnd, bd);
+  put(s->d_ord_l, s->ord_l, one);
+  put(s->d_tick_l, s->tick_l, tk);
+  if (s->upper) {
+    put(s->d_ord_u, s->ord_u, one);
+    put(s->d_tick_u, s->tick_u, tk);
+  }
+  return ok ? BILU_OK : BILU_ERR_CUDA;
+}
+
 int build_schedule_device(const bilu_pattern* p, int32_t target, bool upper, bilu_chunk_schedule* s,
                           ScheduleInputs* in, int32_t least) {
   const int32_t n = p->n;

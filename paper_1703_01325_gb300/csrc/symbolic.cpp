@@ -443,7 +443,7 @@ void ticket_order_lists(int32_t nchunks, const std::vector<int32_t>& prio, const
   // a chunk depends only on chunks earlier in solve order: every chunk is listed
 }
 
-void build_schedule(const bilu_pattern* p, int32_t target, bool upper, bilu_chunk_schedule* s) {
+void build_schedule(const bilu_pattern* p, int32_t target, bool upper, bilu_chunk_schedule* s, int32_t least) {
   const int32_t n = p->n;
   // chunk boundaries from the gaps: r - (last column of L(r)), and the first
   // column of U'(r - 1) - (r - 1)
@@ -455,6 +455,7 @@ void build_schedule(const bilu_pattern* p, int32_t target, bool upper, bilu_chun
   schedule_cuts(n, target, upper, gapl, gapu, s);
   const int32_t nchunks = s->nchunks;
   const int32_t max_len = s->max_len;
+  if (nchunks < least) return;
   std::vector<int32_t> chunk_of((size_t)n);
   for (int32_t c = 0; c < nchunks; ++c)
     for (int32_t i = s->bnd[c]; i < s->bnd[c + 1]; ++i) chunk_of[i] = c;

@@ -89,3 +89,20 @@ def test_failed_reschedule_leaves_all_old_schedules(libbilu):
         assert torch.equal(_apply_of(P), x)
     finally:
         B.bilu_set_trisolve_chunk(0)
+
+
+@pytest.mark.parametrize("dims,k,allocs", [((16, 16, 8), 1, 3), ((8, 6, 5), 0, 2), ((8, 8, 6), 2, 2)])
+def test_small_host_patterns_take_the_host_builder(libbilu, dims, k, allocs):
+    """Small patterns completed on the host need one allocation per schedule (general, factorization and, for lines
+    of 16 rows and more, the second one), and run as the same pattern completed on the device."""
+    rp, ci = grid_pattern(*dims, 7)
+    n = int(np.prod(dims))
+    h, g = B.bilu_symbolic(n, rp, ci, k), B.bilu_symbolic_gpu(n, rp, ci, k).upload()
+    B.bilu_test_fail_alloc(1, allocs)
+    h.upload()
+    B.bilu_test_fail_alloc(0)
+    assert (h.schedule_info(), h.apply_info(3)) == (g.schedule_info(), g.apply_info(3))
+    gen = torch.Generator().manual_seed(1)
+    F = (torch.rand(h.factor_bytes(3) // 8, generator=gen, dtype=torch.float64) * 0.01).cuda()
+    r = torch.rand(3 * n, generator=gen, dtype=torch.float64).cuda()
+    assert torch.equal(B.bilu_apply(h, 3, F, r), B.bilu_apply(g, 3, F, r))
