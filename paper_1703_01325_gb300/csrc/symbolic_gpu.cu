@@ -744,8 +744,9 @@ extern "C" int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_
   if (row_ptr[0] != 0 || row_ptr[n] < n) return BILU_ERR_PATTERN;  // each row holds its diagonal
   // Ascending row pointers on the host, before row_ptr[n] says how many columns
   // are read: col_idx holds no more than the row pointers address.
-  for (int32_t i = 0; i < n; ++i)
-    if (row_ptr[i + 1] < row_ptr[i]) return BILU_ERR_PATTERN;
+  int descends = 0;  // no early exit: the loop runs as vectors
+  for (int32_t i = 0; i < n; ++i) descends |= row_ptr[i + 1] < row_ptr[i];
+  if (descends) return BILU_ERR_PATTERN;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t nnz_a = row_ptr[n];
   const int cap = row_capacity;
