@@ -495,6 +495,11 @@ void launch_tri_k(const TriArgs<TV, RT>& a, size_t smem, cudaStream_t s) {
 // the other lanes' next pass (27-point ILU(2): b = 3 5871 / 6962, b = 2 4676 /
 // 5373), and so it does in FP32 rows of several passes over eight or more
 // groups (b = 4 ILU(2) 849 / 884; b = 5 ILU(1) 551 / 504, b = 8 ILU(2) 1113 / 917).
+// In FP32, where the pipe is not scarce, rows of one pass gain from it while they
+// are spread over at most eight groups of several components (60x60x40, b = 3
+// ILU(0) 230 / 223, b = 2 ILU(1) 376 / 367) and lose when every lane or every
+// second one may be waiting (b = 1: 27-point ILU(1) 625 / 722, ILU(2) 543 / 610,
+// ILU(1) 361 / 388; b = 2 ILU(2), 16 groups, 560 / 568).
 template <int B, bool UPPER, typename TV, int W, int GE, typename RT>
 void launch_tri(const TriArgs<TV, RT>& a, int32_t max_blocks, size_t smem, cudaStream_t s) {
   const int passes = (max_blocks + GE - 1) / GE;
@@ -503,7 +508,7 @@ void launch_tri(const TriArgs<TV, RT>& a, int32_t max_blocks, size_t smem, cudaS
     if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
     if (passes <= 4) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, false>(a, smem, s);
   } else {
-    if (passes == 1) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
+    if (passes == 1) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, B != 1 && GE <= 8>(a, smem, s);
     if constexpr (B >= 5)
       if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, true, true>(a, smem, s);
   }
