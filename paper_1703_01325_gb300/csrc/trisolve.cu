@@ -86,13 +86,19 @@ int device_sm_count() {
 // Rows of more than eight blocks on smaller grids: one line, whose level has a
 // row for one warp while the others fetch theirs (27-point 80x80x40 ILU(2) b =
 // 3: 7.3 ms with two lines, 6.1 with one; 64x64x32 ILU(1): 2.57, 2.42).
+constexpr int kNarrow = 8;
+
+int32_t size_chunk_target(const bilu_pattern* p) {
+  return (int32_t)std::max(32LL, std::min(256LL, (long long)p->n / (10LL * device_sm_count())));
+}
+
 int32_t auto_solve_chunk_target(const bilu_pattern* p) {
-  const long long t = (long long)p->n / (10LL * device_sm_count());
+  const int32_t t = size_chunk_target(p);
   if (p->line_len >= 16 && p->line_len <= 192) {
-    if (t >= 256) return 2 * p->line_len;
-    if (std::max(p->max_l, p->max_u) > 8) return p->line_len;
+    if (t == 256) return 2 * p->line_len;
+    if (std::max(p->max_l, p->max_u) > kNarrow) return p->line_len;
   }
-  return (int32_t)std::max(32LL, std::min(256LL, t));
+  return t;
 }
 
 // The schedule of rows that take one pass over the groups, on grids too small
@@ -109,23 +115,30 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // of step (grids whose lines each lost up to a share of their cells, ILU(1) b = 3,
 // general schedule / two lines: 40x40x20, a fifth 272 / 381, half 266 / 553;
 // 30x30x30, 0.3 283 / 377; 64x64x32, 0.3 470 / 472, 0.6 563 / 536).
+// Wider rows have one line per chunk in the general schedule, which suits FP64 but
+// not FP32 rows of at most two passes (FP32, one line / two: 16x30x30 ILU(2) b = 3
+// 517 / 483, b = 4 535 / 483, 16x60x60 27-point ILU(1) b = 1 1040 / 848; three passes
+// and more 28x40x20 ILU(2) b = 5 551 / 571, 16x30x30 27-point b = 3 952 / 1022).
+// Where the size rule alone would cut two lines they get those.
 constexpr int kPairLine = 64;
 
 int32_t pair_chunk_target(const bilu_pattern* p) {
-  const int widest = std::max(p->max_l, p->max_u);
-  if (trisolve_config().chunk > 0 || p->line_len < 16 || p->line_len > 192 || widest > 8 ||
-      (long long)p->line_starts * p->line_len != p->n ||
-      (p->line_len > kPairLine && widest <= 4) || auto_solve_chunk_target(p) == 2 * p->line_len)
+  const int widest = std::max(p->max_l, p->max_u), line = p->line_len;
+  if (trisolve_config().chunk > 0 || line < 16 || line > 192 || (long long)p->line_starts * line != p->n ||
+      auto_solve_chunk_target(p) == 2 * line)
     return 0;
-  return 2 * p->line_len;
+  const int32_t t = size_chunk_target(p);
+  if (widest > kNarrow ? 2 * t < 3 * line || 2 * t > 5 * line : line > kPairLine && widest <= 4) return 0;
+  return 2 * line;
 }
 
 int32_t pair_least_chunks(const bilu_pattern* p) { return (int32_t)std::ceil(p->n / (2.1 * p->line_len)); }
 
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32) {
-  const bool one_pass = std::max(p->max_l, p->max_u) <= groups_for(b);
-  const bool lines = !f32 || p->line_len <= kPairLine;
-  return one_pass && lines && p->pair.d_mem && trisolve_config().warps <= 4 ? p->pair : p->solve;
+  const int widest = std::max(p->max_l, p->max_u), groups = groups_for(b);
+  const bool two_lines = widest > kNarrow ? f32 && widest <= 2 * groups
+                                          : widest <= groups && (!f32 || p->line_len <= kPairLine);
+  return two_lines && p->pair.d_mem && trisolve_config().warps <= 4 ? p->pair : p->solve;
 }
 
 // Rows of many passes: eight warps per CTA, so that a level's rows have been

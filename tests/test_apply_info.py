@@ -41,6 +41,8 @@ def test_warps_that_are_set_are_used(libbilu):
     ((30, 30, 30), 5, 0, 60, 60),
     ((30, 30, 30), 5, 1, 32, 32),    # two passes over four groups: the general schedule
     ((30, 30, 30), 3, 2, None, None),  # rows of more than eight blocks: no second schedule
+    ((16, 30, 30), 3, 2, None, 32),  # wide rows of two passes, FP32: the two lines of the size rule
+    ((16, 30, 30), 5, 2, None, None),  # three passes
     ((70, 30, 10), 3, 1, 140, 32),   # lines above 64 rows: FP64 only
     ((70, 30, 10), 3, 0, 32, 32),    # and not for rows of four blocks and fewer
 ])
