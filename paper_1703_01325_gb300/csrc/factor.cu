@@ -57,22 +57,44 @@ __global__ void factor_init_kernel(int32_t* header, int32_t* done, int32_t n) {
 // anything is waited for.  8 warps per CTA: twice the chunks in flight of one
 // 16-warp CTA for the same warps (measured 4-13 % faster with 256-row chunk
 // targets).
-template <int B>
+// LC: a 27-point ILU(1) row has 25 entries; a batch below that takes each pivot in
+// slices, so it holds one such row and more, as far as the CTAs per SM allow
+// (b = 5 FP32 128x16x8 27-point with 16 / 42 entries: 12.2 / 9.7 ms; b = 3 FP32
+// 160x40x20 with 48 / 96: 11.2 / 9.2; b = 1 FP64 12x60x60 with 64 / 128: 18.0 /
+// 15.6; with 256, 7-point b = 1 2.30 / 2.54).
+// MINB: CTAs per SM the registers are cut for, 0 the compiler's choice: FP32 b = 2
+// otherwise takes 80 registers (96x96x48 ILU(0): 1400 us, with 58 1267), and FP64
+// b >= 6 does better with the 128 there are (160x20x20 27-point b = 6 36.6 -> 34.7 ms).
+template <int B, typename TV>
 struct FactorCap {
+  static constexpr bool kSingle = sizeof(TV) == 4;
   static constexpr int W = 8;  // warps per CTA
   static constexpr int RC = B <= 4 ? 64 : (B <= 6 ? 32 : 24);
-  static constexpr int LC = B <= 2 ? 64 : B == 3 ? 48 : B == 4 ? 32 : B <= 6 ? 16 : 12;
+  static constexpr int LC = B == 1 ? 128
+                            : B == 2 ? 96
+                            : kSingle ? (B == 3 ? 96 : B == 4 ? 64 : B <= 6 ? 42 : B == 7 ? 28 : 20)
+                                      : (B == 3 ? 64 : B == 4 ? 32 : B <= 6 ? 28 : 16);
+  static constexpr int MINB = B == 2 && kSingle ? 4 : B >= 6 && !kSingle ? 2 : 0;
   static constexpr int KC = B <= 4 ? 16 : 6;  // pivot blocks D_p^{-1} held at once
   static constexpr int WVAL = (LC + KC + 1) * B * B;  // values per warp beside the staged row
   static constexpr int WINT = 2 * LC + 2 * 34;        // ints per warp beside the row's columns
 };
 
 // rc: rows of up to rc blocks are staged (at most RC; the widest row of the
-// pattern if that is less).
+// pattern if that is less).  For b >= 5 none are where the mean row is longer than
+// RC: the buffer would cost a CTA per SM and hold boundary rows only (FP64 b = 8
+// 128x16x8 27-point 28.7 / 25.7 ms).
+template <int B, typename TV>
+int staged_rows(const bilu_pattern* p) {
+  constexpr int RC = FactorCap<B, TV>::RC;
+  if (B >= 5 && p->cnt_p > (long long)p->n * RC) return 0;
+  return std::min(RC, p->max_l + 1 + p->max_u);
+}
+
 template <int B, typename TV>
 size_t factor_smem_bytes(int chunk, int rc) {
-  return (size_t)FactorCap<B>::W * (FactorCap<B>::WVAL + rc * B * B) * sizeof(TV) +
-         ((size_t)2 * chunk + (size_t)FactorCap<B>::W * (FactorCap<B>::WINT + rc)) * sizeof(int);
+  return (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WVAL + rc * B * B) * sizeof(TV) +
+         ((size_t)2 * chunk + (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WINT + rc)) * sizeof(int);
 }
 
 // Whether a value is finite, and the order of magnitudes, on the integer pipes
@@ -140,13 +162,13 @@ __device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
 // blocks of all pivots that are finished are fetched in one round trip, with
 // only what depends on the last pivots left once those arrive.
 template <int B, typename TV>
-__global__ void __launch_bounds__(FactorCap<B>::W * 32) factor_kernel(
+__global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MINB) factor_kernel(
     int32_t n, int32_t chunk, int32_t rc, int32_t nchunks, const int32_t* __restrict__ bnd,
     const int32_t* __restrict__ ord, const int32_t* __restrict__ tick,
     const int32_t* __restrict__ lrp, const int32_t* __restrict__ lci,
     const int32_t* __restrict__ urp, const int32_t* __restrict__ uci, TV* f, long long nnz_l,
     int32_t* header, int32_t* done, long long spin_ns) {
-  using Cap = FactorCap<B>;
+  using Cap = FactorCap<B, TV>;
   constexpr int BB = B * B;
   constexpr int H = (BB + 31) / 32;
   constexpr int LC = Cap::LC, KC = Cap::KC;
@@ -332,10 +354,10 @@ __global__ void __launch_bounds__(FactorCap<B>::W * 32) factor_kernel(
           run = min(min(run, nfit - x), KC);
           // their D_p^{-1} and matching U_pj, all loads in flight together
           const int m0 = moff[x], mv = (moff[x + run] - m0) * BB, dv = run * BB;
-          constexpr int ND = (KC * BB + 31) / 32 < 5 ? (KC * BB + 31) / 32 : 5;
-          constexpr int NU = 6;
-          for (int e0 = 0; e0 < dv || e0 < mv; e0 += 32 * (ND < NU ? ND : NU)) {
-            constexpr int NB = ND < NU ? ND : NU;
+          // (eight a lane for large blocks, whose batches take many rounds)
+          constexpr int NMAX = B >= 6 ? 8 : 5;
+          constexpr int NB = (KC * BB + 31) / 32 < NMAX ? (KC * BB + 31) / 32 : NMAX;
+          for (int e0 = 0; e0 < dv || e0 < mv; e0 += 32 * NB) {
             TV tu[NB], td[NB];
 #pragma unroll
             for (int h = 0; h < NB; ++h) {
@@ -388,14 +410,40 @@ __global__ void __launch_bounds__(FactorCap<B>::W * 32) factor_kernel(
             }
             // A_ij <- A_ij - A_ip U_pj
             const int mb = moff[x + y], cnt = (moff[x + y + 1] - mb) * BB;
-            for (int wk = lane; wk < cnt; wk += 32) {
-              const int sidx = wk / BB, e = wk - sidx * BB;
+            auto term = [&](int sidx, int e) {
               const int r = e % B, cc = e / B;
               const TV* const upj = ub + (mb - m0 + sidx) * BB + cc * B;
               TV s = TV(0);
 #pragma unroll
               for (int m = 0; m < B; ++m) s = fma(aip[m * B + r], upj[m], s);
-              blk(mdst[mb + sidx])[e] -= s;
+              return s;
+            };
+            if (B >= 6 && !staged) {
+              // in place: two elements a lane at a time, both read before either is
+              // written (a pivot's matches are different blocks); one at a time is a
+              // chain of round trips (b = 7 FP32 160x20x20 27-point 34.4 / 27.6 ms)
+              for (int w0 = lane; w0 < cnt; w0 += 64) {
+                const int w1 = w0 + 32;
+                const int s0i = w0 / BB, e0 = w0 - s0i * BB;
+                TV* const at0 = blk(mdst[mb + s0i]) + e0;
+                const TV was0 = *at0;
+                if (w1 < cnt) {
+                  const int s1i = w1 / BB, e1 = w1 - s1i * BB;
+                  TV* const at1 = blk(mdst[mb + s1i]) + e1;
+                  const TV was1 = *at1;
+                  const TV t0 = term(s0i, e0), t1 = term(s1i, e1);
+                  *at0 = was0 - t0;
+                  *at1 = was1 - t1;
+                } else {
+                  *at0 = was0 - term(s0i, e0);
+                }
+              }
+            } else {
+              for (int wk = lane; wk < cnt; wk += 32) {
+                const int sidx = wk / BB, e = wk - sidx * BB;
+                const TV s = term(sidx, e);
+                blk(mdst[mb + sidx])[e] -= s;
+              }
             }
             __syncwarp();
           }
@@ -508,19 +556,18 @@ int launch_factor_t(const bilu_pattern* p, int32_t b, TV* f, int32_t* header, in
   const int nchunks = p->fact.nchunks;
   const long long spin = trisolve_config().spin_ns;
   BILU_DISPATCH_B(b, {
-    // rows of the pattern are at most max_l + 1 + max_u blocks wide
-    const int rc = std::min(FactorCap<B>::RC, p->max_l + 1 + p->max_u);
+    const int rc = staged_rows<B, TV>(p);
     const size_t smem = factor_smem_bytes<B, TV>(chunk, rc);
     static LaunchCache cache;
     const int per_sm = cache.ctas_per_sm(current_device(), smem, [](size_t bytes) {
       cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
       int q = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, factor_kernel<B, TV>, FactorCap<B>::W * 32, bytes);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, factor_kernel<B, TV>, FactorCap<B, TV>::W * 32, bytes);
       return q;
     });
     const int grid = std::max(1, std::min(nchunks, per_sm * sms));
     ProfScope ps(BILU_PROF_FACTOR, stream);
-    factor_kernel<B, TV><<<grid, FactorCap<B>::W * 32, smem, s>>>(n, chunk, rc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
+    factor_kernel<B, TV><<<grid, FactorCap<B, TV>::W * 32, smem, s>>>(n, chunk, rc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
                                                             p->d_urp, p->d_uci, f, p->nnz_l(), header, done,
                                                             spin);
   });
