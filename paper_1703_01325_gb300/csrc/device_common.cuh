@@ -194,17 +194,6 @@ __device__ __forceinline__ void st_release_cta_shared_s32(int* p, int v) {
   asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 
-// Wait until a shared-memory flag of this CTA equals `want` (acquire, CTA
-// scope); false if the wait was abandoned.  The abort word (a global load)
-// and the clock are consulted every 1024 polls only.
-__device__ __forceinline__ bool wait_local_flag(const int* flag, int want, Waiter& w) {
-  w.t0 = 0;
-  for (unsigned it = 1;; ++it) {
-    if (ld_acquire_cta_shared_s32(flag) == want) return true;
-    if (w.give_up(it, 1023u)) return false;
-  }
-}
-
 // double -> float, rounded to nearest even, on the integer pipes: rebias the
 // exponent, keep 23 mantissa bits and round on the 29 dropped ones (round up
 // when the dropped bits plus the kept last bit exceed half; a carry into the

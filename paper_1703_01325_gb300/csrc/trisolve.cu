@@ -515,17 +515,24 @@ void launch_tri_k(const TriArgs<TV, RT>& a, size_t smem, cudaStream_t s) {
 // ILU(1) 361 / 388; b = 2 ILU(2), 16 groups, 560 / 568).
 template <int B, bool UPPER, typename TV, int W, int GE, typename RT>
 void launch_tri(const TriArgs<TV, RT>& a, int32_t max_blocks, size_t smem, cudaStream_t s) {
-  const int passes = (max_blocks + GE - 1) / GE;
-  const bool join = passes <= (W == 4 ? 4 : 3);
-  if constexpr (sizeof(TV) == 8) {
-    if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
-    if (passes <= 4) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, false>(a, smem, s);
+  constexpr bool kDouble = sizeof(TV) == 8;
+  constexpr bool kJoinOne = kDouble || (B != 1 && GE <= 8);
+  if constexpr (GE < groups_for(B)) {  // chosen for rows of one pass only
+    launch_tri_k<B, UPPER, TV, W, GE, RT, false, kJoinOne>(a, smem, s);
   } else {
-    if (passes == 1) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, B != 1 && GE <= 8>(a, smem, s);
-    if constexpr (B >= 5)
-      if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, true, true>(a, smem, s);
+    const int passes = (max_blocks + GE - 1) / GE;
+    const bool join = passes <= (W == 4 ? 4 : 3);
+    if constexpr (kDouble) {
+      if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, true>(a, smem, s);
+      if constexpr (W > 4)
+        if (passes == 4) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, false>(a, smem, s);
+    } else {
+      if (passes == 1) return launch_tri_k<B, UPPER, TV, W, GE, RT, false, kJoinOne>(a, smem, s);
+      if constexpr (B >= 5)
+        if (join) return launch_tri_k<B, UPPER, TV, W, GE, RT, true, true>(a, smem, s);
+    }
+    launch_tri_k<B, UPPER, TV, W, GE, RT, true, false>(a, smem, s);
   }
-  launch_tri_k<B, UPPER, TV, W, GE, RT, true, false>(a, smem, s);
 }
 
 // The fewest groups (a power of two, at least groups_for(B) / 4) that hold
