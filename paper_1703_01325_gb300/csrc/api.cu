@@ -31,13 +31,14 @@ int build_schedules(bilu_pattern* p) {
   ScheduleInputs in;
   bilu_chunk_schedule solve, pair, fact;
   int st = make_schedule(p, &solve, solve_chunk_target(p), true, &in);
+  const int32_t target = st == BILU_OK ? pair_chunk_target(p) : 0;
+  if (target > 0 && make_schedule(p, &pair, target, true, &in, pair_least_chunks(p)) != BILU_OK) cudaGetLastError();
   if (st == BILU_OK && !p->is_transpose) st = make_schedule(p, &fact, factor_chunk_target(p), false, &in);
   if (st != BILU_OK) {
     free_schedule(&solve);
+    free_schedule(&pair);
     return st;
   }
-  const int32_t target = pair_chunk_target(p);
-  if (target > 0 && make_schedule(p, &pair, target, true, &in, pair_least_chunks(p)) != BILU_OK) cudaGetLastError();
   std::swap(p->solve, solve);
   std::swap(p->pair, pair);
   std::swap(p->fact, fact);

@@ -177,13 +177,13 @@ __global__ void __launch_bounds__(128) chunk_preds_kernel(int32_t nchunks, const
     const int lc = UPPER ? nchunks - 1 - c : c;
     const int lo = bnd[lc], hi = bnd[lc + 1];
     int pm = INT_MAX;
-    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+    bool full = false;  // this thread found one predecessor too many
+    for (int i = lo + threadIdx.x; i < hi && !full; i += blockDim.x) {
       pm = min(pm, lvl[i]);
       int a = 0, z = 0;  // rows of the chunk of the previous entry: most entries fall in it again
-      for (int t = rpv[i]; t < rpv[i + 1]; ++t) {
+      for (int t = rpv[i]; t < rpv[i + 1] && !full; ++t) {
         const int j = civ[t];
         if ((j >= lo && j < hi) || (j >= a && j < z)) continue;
-        if (*reinterpret_cast<volatile int*>(&s_n) > kMaxPreds) break;
         const int lj = chunk_of_row(bnd, nchunks, j);
         a = bnd[lj];
         z = bnd[lj + 1];
@@ -191,7 +191,10 @@ __global__ void __launch_bounds__(128) chunk_preds_kernel(int32_t nchunks, const
         unsigned h = (unsigned)cj * 2654435761u >> 24;
         for (int tries = 0;; ++tries) {
           const int was = tries < 4 * kMaxPreds ? atomicCAS(&set[h], -1, cj) : cj;
-          if (was == -1 && atomicAdd(&s_n, 1) >= kMaxPreds) *over = 1;
+          if (was == -1 && atomicAdd(&s_n, 1) >= kMaxPreds) {
+            *over = 1;
+            full = true;
+          }
           if (was == -1 || was == cj) break;
           h = (h + 1) % (4 * kMaxPreds);
         }
