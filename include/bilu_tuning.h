@@ -64,7 +64,8 @@ int32_t bilu_get_factor_chunk(void);
 int32_t bilu_auto_factor_chunk(const bilu_pattern* p);
 
 /* Warps per CTA in the triangular solves: 0 (the default) picks 8 for rows of 40
- * blocks or more that take at least four passes of a warp and 4 for all others;
+ * blocks or more that take at least four passes of a warp (in double, while the
+ * rows per level leave enough chunks resident) and 4 for all others;
  * 4, 8 or 16 fixes it; else BILU_ERR_ARG.  More warps per chunk give each row more time to fetch its
  * operands ahead of its dependencies.  Applies to the next launch. */
 int bilu_set_trisolve_warps(int32_t warps);

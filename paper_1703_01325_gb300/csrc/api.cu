@@ -516,7 +516,7 @@ extern "C" int bilu_apply_info(const bilu_pattern* p, int32_t b, int32_t f32, in
   if (!p || !valid_b(b)) return BILU_ERR_ARG;
   const bilu_chunk_schedule& s = apply_schedule(p, b, f32 != 0);
   if (rows) *rows = s.d_mem ? s.chunk : 0;
-  if (warps) *warps = apply_warps(p, b);
+  if (warps) *warps = apply_warps(p, b, f32 != 0);
   return BILU_OK;
 }
 

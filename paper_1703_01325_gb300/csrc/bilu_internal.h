@@ -10,8 +10,8 @@
 #include "../../include/bilu.h"
 #include "../../include/bilu_tuning.h"
 
-// Sync-free schedule for one target chunk size (symbolic.cpp builds it,
-// trisolve.cu uploads it): rows cut into chunks of consecutive rows, chunk c
+// Sync-free schedule for one target chunk size (built by schedule_gpu.cu, or by
+// symbolic.cpp for small host patterns): rows cut into chunks of consecutive rows, chunk c
 // = rows [bnd[c], bnd[c+1]) (walked in ascending chunk order for L, descending
 // for U'); ord_l / ord_u list each chunk's rows by local dependency level at
 // the positions of the chunk's rows; tick_l / tick_u give the chunk each
@@ -120,16 +120,16 @@ TrisolveConfig& trisolve_config();
 // The chunk targets in effect for a pattern of n block rows: the configured
 // ones, or (0) n / (10 * SMs) in [32, 256] for the solves and n / (2 * SMs)
 // in [64, 256] for the factorization -- enough chunks to fill the GPU --
-// except with a detected line length L: 2 L for the solves of large grids
-// (16 <= L <= 192), L to 3 L by row width for the factorization (16 <= L <=
-// 128).
+// except with a detected line length L: 2 L for the solves of large grids, L for
+// wide rows on smaller ones (16 <= L <= 192), L to 3 L by row width for the
+// factorization (16 <= L <= 128).
 int32_t solve_chunk_target(const bilu_pattern* p);
 int32_t auto_solve_chunk_target(const bilu_pattern* p);  // the rule alone
 int32_t pair_chunk_target(const bilu_pattern* p);
 int32_t pair_least_chunks(const bilu_pattern* p);  // fewer would hold more than two lines each
 // What an apply runs on: the schedule, and the warps per CTA of its sweeps.
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32);
-int apply_warps(const bilu_pattern* p, int32_t b);
+int apply_warps(const bilu_pattern* p, int32_t b, bool f32);
 int32_t factor_chunk_target(const bilu_pattern* p);
 int32_t auto_factor_chunk_target(const bilu_pattern* p);  // the rule alone
 

@@ -104,8 +104,10 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // The schedule of rows that take one pass over the groups, on grids too small
 // for two lines per chunk above: 0 (none), or two lines.  Such rows are done
 // within a level of two lines, and half the hand-offs between chunks go (apply,
-// us, 1 line / 2 lines: 64x64x32 ILU(1) b = 3 523 / 488, 30x30x30 323 / 285,
-// 61x47x33 ILU(0) b = 5 310 / 293, 150x30x20 ILU(1) b = 4 465 / 394); rows of
+// us, general schedule / two lines: 64x1000x1 ILU(1) b = 3 2892 / 2335, 40x200x5
+// 645 / 601, 30x30x30 ILU(0) b = 5 182 / 170, 64x64x32 ILU(0) b = 3 290 / 281; no
+// gain since the lanes are joined, see JOIN below, 30x30x30 ILU(1) b = 3 285 / 287,
+// and a small loss 64x64x32 ILU(1) b = 4 482 / 494, FP32 403 / 398); rows of
 // two passes are not (b = 5 ILU(1) 883 / 967, b = 6 874 / 937), nor grids whose
 // few lines per plane leave chunks of three (100x9x60 ILU(0) b = 8: 379 / 405;
 // pair_least_chunks).  Two long lines hold a chunk too long where a row is quick:
@@ -143,12 +145,29 @@ const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool
 
 // Rows of many passes: eight warps per CTA, so that a level's rows have been
 // fetched when their turn comes (apply, ms, 4 / 8 warps: 27-point ILU(2) b = 2
-// 128x128x40 6.19 / 4.87, b = 3 80x80x40 6.09 / 5.88, FP32 5.06 / 4.59).  Rows
+// 128x128x40 6.46 / 4.87, b = 3 80x80x40 6.09 / 5.88, FP32 5.07 / 4.60).  Rows
 // of fewer blocks or passes are not faster (27-point ILU(1) b = 3 2.42 / 2.45;
 // 27-point ILU(2) b = 1, two passes, 1.81 / 1.86).
-int apply_warps(const bilu_pattern* p, int32_t b) {
+// In FP64 eight-warp CTAs also leave fewer chunks resident (registers: 3 per SM at b
+// = 2 and 3, 2 up to b = 6, 1 above; four-warp ones 8, 5, 5, 4, 4, 3, 3), and every
+// line of a grid advances a row per level: where the rows per level, which are the
+// lines to keep going, come near the lines that fit, four warps win.  Rows per level
+// over lines resident with eight warps, and 4 / 8 warps, 27-point ILU(2): b = 3
+// 160x160x80 1.09 16.1 / 17.7, 160x160x40 0.79 10.7 / 10.5, 128x128x80 0.76 14.2 /
+// 13.1; b = 4 128x128x80 1.13 22.9 / 24.6, 128x128x40 0.86 15.0 / 14.4; b = 5 96x96x96
+// 0.73 41.8 / 37.5; b = 6 80x80x40 0.83 20.6 / 21.0; b = 8 80x80x40 1.65 21.9 / 34.9,
+// 60x50x40 0.89 18.6 / 19.3, 40x40x20 0.42 10.2 / 9.8; b = 2, whose rows take four
+// passes, 160x160x80 1.09 10.8 / 8.9, 160x160x40 one line 1.58 6.5 / 6.6.
+int apply_warps(const bilu_pattern* p, int32_t b, bool f32) {
   const int set = trisolve_config().warps, widest = std::max(p->max_l, p->max_u);
-  return set > 0 ? set : widest >= 40 && widest > 3 * groups_for(b) ? 8 : 4;
+  if (set > 0) return set;
+  if (widest < 40 || widest <= 3 * groups_for(b)) return 4;
+  if (f32) return 8;
+  const int chunk = p->solve.chunk > 0 ? p->solve.chunk : solve_chunk_target(p);
+  const int lines = p->line_len > 0 ? std::max(1, (chunk + p->line_len / 2) / p->line_len) : 1;
+  const int ctas = b == 1 ? 5 : b <= 3 ? 3 : b <= 6 ? 2 : 1;
+  const double share = b <= 2 ? 1.5 : b <= 5 ? 0.87 : 0.8;
+  return p->n <= share * lines * ctas * device_sm_count() * std::max(p->nlev_l, p->nlev_u) ? 8 : 4;
 }
 
 int32_t solve_chunk_target(const bilu_pattern* p) {
@@ -609,7 +628,7 @@ int launch_apply_t(const bilu_pattern* p, int32_t b, const TV* f, const double* 
     ProfScope ps(BILU_PROF_APPLY_PREP, stream);
     apply_prep_kernel<TV><<<prep_blocks, 256, 0, s>>>(y, xs, m, header, stop);
   }
-  const int warps = apply_warps(p, b);
+  const int warps = apply_warps(p, b, sizeof(TV) == 4);
   BILU_DISPATCH_B(b, {
     if (warps == 16)
       launch_solves<B, TV, 16>(p, sch, L, Dinv, U, r, y, xs, header, cfg, stop, stream);

@@ -27,7 +27,7 @@ def test_warps_that_are_set_are_used(libbilu):
     P = B.bilu_symbolic(504, rp, ci, 2)
     try:
         B.bilu_set_trisolve_warps(0)
-        assert [P.apply_info(b)["warps"] for b in (1, 2, 3, 8)] == [4, 8, 8, 8]
+        assert [P.apply_info(b, f32=True)["warps"] for b in (1, 2, 3, 8)] == [4, 8, 8, 8]
         for w in (4, 8, 16):
             B.bilu_set_trisolve_warps(w)
             assert [P.apply_info(b)["warps"] for b in (1, 3, 8)] == [w] * 3
@@ -67,6 +67,19 @@ def test_which_schedule(libbilu, dims, b, k, f64, f32):
         B.bilu_set_trisolve_chunk(old)
     assert P.apply_info(b)["rows"] == P.apply_info(b, f32=True)["rows"] == general
     assert torch.equal(B.bilu_apply(P, b, F, rhs), x) and torch.equal(B.bilu_apply_f32(P, b, F32, rhs), x32)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dims,wide,narrow", [((60, 50, 40), (2, 3, 4, 5, 6), (8,)), ((40, 40, 20), (2, 3, 4, 5, 6, 7, 8), ())])
+def test_eight_warps_while_enough_lines_are_resident(libbilu, dims, wide, narrow):
+    """27-point ILU(2) rows: 136 and 64 rows per level, on 152 SMs with three, two (b >= 4) or one (b >= 7)
+    eight-warp CTA each."""
+    torch.cuda.set_device(0)
+    B.bilu_set_trisolve_warps(0)
+    n = dims[0] * dims[1] * dims[2]
+    P = B.bilu_symbolic_gpu(n, *grid_pattern(*dims, 27), 2).upload()
+    assert all(P.apply_info(b)["warps"] == 8 for b in wide) and all(P.apply_info(b)["warps"] == 4 for b in narrow)
+    assert all(P.apply_info(b, f32=True)["warps"] == 8 for b in wide + narrow)
 
 
 @pytest.mark.gpu
