@@ -26,8 +26,8 @@ extern "C" {
  * where the widest row of L or U' has more than 8 blocks, and otherwise a
  * second schedule of 2 L, if every line has L rows, for rows that take one pass
  * of a warp (L > 64: in double only, and of more than 4 blocks) or, in single,
- * for rows of more than 8 blocks and at most two passes where n / (10 * SMs) is
- * nearest to 2 L; 1 <= rows <=
+ * for rows of more than 8 blocks and at most two passes, in double for b >= 7 with
+ * more rows per level than 3 SMs, where n / (10 * SMs) is nearest to 2 L; 1 <= rows <=
  * 1024 fixes the target (and leaves out the second schedule);
  * other values: BILU_ERR_ARG.  Takes effect for a pattern at its next
  * bilu_pattern_upload or bilu_pattern_schedule (the set-up calls that build

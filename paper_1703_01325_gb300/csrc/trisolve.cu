@@ -121,7 +121,11 @@ int32_t auto_solve_chunk_target(const bilu_pattern* p) {
 // not FP32 rows of at most two passes (FP32, one line / two: 16x30x30 ILU(2) b = 3
 // 517 / 483, b = 4 535 / 483, 16x60x60 27-point ILU(1) b = 1 1040 / 848; three passes
 // and more 28x40x20 ILU(2) b = 5 551 / 571, 16x30x30 27-point b = 3 952 / 1022).
-// Where the size rule alone would cut two lines they get those.
+// Where the size rule alone would cut two lines they get those, and so do FP64 rows
+// of b >= 7, three chunks per SM, with more rows per level than lines would be
+// resident one by one (27-point ILU(1) b = 8, rows per level over resident lines, one
+// line / two: 120x80x35 1.11 10.95 / 9.83 ms, 60x100x60 0.89 12.35 / 12.53, 64x64x64
+// 0.70 10.2 / 11.5; b = 6, four chunks, 120x80x35 0.83 8.87 / 8.78).
 constexpr int kPairLine = 64;
 
 int32_t pair_chunk_target(const bilu_pattern* p) {
@@ -138,7 +142,9 @@ int32_t pair_least_chunks(const bilu_pattern* p) { return (int32_t)std::ceil(p->
 
 const bilu_chunk_schedule& apply_schedule(const bilu_pattern* p, int32_t b, bool f32) {
   const int widest = std::max(p->max_l, p->max_u), groups = groups_for(b);
-  const bool two_lines = widest > kNarrow ? f32 && widest <= 2 * groups
+  const bool two_lines = widest > kNarrow ? (f32 ? widest <= 2 * groups
+                                                 : b >= 7 && p->n > 3LL * device_sm_count() *
+                                                                        std::max(p->nlev_l, p->nlev_u))
                                           : widest <= groups && (!f32 || p->line_len <= kPairLine);
   return two_lines && p->pair.d_mem && trisolve_config().warps <= 4 ? p->pair : p->solve;
 }

@@ -43,6 +43,7 @@ def test_warps_that_are_set_are_used(libbilu):
     ((30, 30, 30), 3, 2, None, None),  # rows of more than eight blocks: no second schedule
     ((16, 30, 30), 3, 2, None, 32),  # wide rows of two passes, FP32: the two lines of the size rule
     ((16, 30, 30), 5, 2, None, None),  # three passes
+    ((16, 30, 30), 8, 2, None, None),  # few rows per level
     ((70, 30, 10), 3, 1, 140, 32),   # lines above 64 rows: FP64 only
     ((70, 30, 10), 3, 0, 32, 32),    # and not for rows of four blocks and fewer
 ])
@@ -67,6 +68,18 @@ def test_which_schedule(libbilu, dims, b, k, f64, f32):
         B.bilu_set_trisolve_chunk(old)
     assert P.apply_info(b)["rows"] == P.apply_info(b, f32=True)["rows"] == general
     assert torch.equal(B.bilu_apply(P, b, F, rhs), x) and torch.equal(B.bilu_apply_f32(P, b, F32, rhs), x32)
+
+
+@pytest.mark.gpu
+def test_large_blocks_with_many_rows_per_level(libbilu):
+    """120x80x35 ILU(2): 565 rows per level, more than the 456 lines that three CTAs on each of 152 SMs hold, where
+    the size rule cuts two lines: FP64 rows of b >= 7 and FP32 rows of two passes run on two lines."""
+    torch.cuda.set_device(0)
+    B.bilu_set_trisolve_warps(0)
+    P = B.bilu_symbolic_gpu(336000, *grid_pattern(120, 80, 35, 7), 2).upload()
+    assert P.schedule_info()["solve_rows"] == 120
+    assert [P.apply_info(b)["rows"] for b in (1, 3, 6, 7, 8)] == [120, 120, 120, 240, 240]
+    assert [P.apply_info(b, f32=True)["rows"] for b in (1, 4, 5, 8)] == [240, 240, 120, 120]
 
 
 @pytest.mark.gpu
