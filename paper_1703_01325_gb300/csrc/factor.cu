@@ -53,48 +53,87 @@ __global__ void factor_init_kernel(int32_t* header, int32_t* done, int32_t n) {
 // Row storage of the factor kernel: rows of up to RC blocks are staged in
 // shared memory (per warp); longer rows are worked on in place in global memory
 // through the same slot interface.  A warp takes a row's pivots in batches of
-// up to LC entries of their U rows, whose matches in the row are listed before
+// up to lc entries of their U rows, whose matches in the row are listed before
 // anything is waited for.  8 warps per CTA: twice the chunks in flight of one
 // 16-warp CTA for the same warps (measured 4-13 % faster with 256-row chunk
 // targets).
-// LC: a 27-point ILU(1) row has 25 entries; a batch below that takes each pivot in
-// slices, so it holds one such row and more, as far as the CTAs per SM allow
-// (b = 5 FP32 128x16x8 27-point with 16 / 42 entries: 12.2 / 9.7 ms; b = 3 FP32
-// 160x40x20 with 48 / 96: 11.2 / 9.2; b = 1 FP64 12x60x60 with 64 / 128: 18.0 /
-// 15.6; with 256, 7-point b = 1 2.30 / 2.54).
-// MINB: CTAs per SM the registers are cut for, 0 the compiler's choice: FP32 b = 2
-// otherwise takes 80 registers (96x96x48 ILU(0): 1400 us, with 58 1267), and FP64
-// b >= 6 does better with the 128 there are (160x20x20 27-point b = 6 36.6 -> 34.7 ms).
+// lc (LCMIN to LCMAX, batch_entries): a 27-point ILU(1) row has 25 entries; a batch
+// below that takes each pivot in slices (b = 5 FP32 128x16x8 27-point with 16 / 42
+// entries: 12.2 / 9.6 ms; b = 3 FP32 160x40x20 with 48 / 96: 11.2 / 9.2; b = 1 FP64
+// 12x60x60 with 64 / 128: 18.0 / 15.6; with 256, 7-point b = 1 2.30 / 2.54).
+// MINB: CTAs per SM the registers are cut for, 0 the compiler's choice (80 registers
+// and 9 to 20 words spilled for FP64 b = 2 and FP32 b = 3 and 5, three CTAs): FP32 b =
+// 2 and 4 otherwise take 80 and 94 (96x96x48 ILU(0) 1.40 / 1.27 and 2.29 / 1.92 ms),
+// and FP64 b >= 6 does better with the 128 there are (160x20x20 27-point b = 6 36.6 /
+// 34.7).
 template <int B, typename TV>
 struct FactorCap {
   static constexpr bool kSingle = sizeof(TV) == 4;
   static constexpr int W = 8;  // warps per CTA
   static constexpr int RC = B <= 4 ? 64 : (B <= 6 ? 32 : 24);
-  static constexpr int LC = B == 1 ? 128
-                            : B == 2 ? 96
-                            : kSingle ? (B == 3 ? 96 : B == 4 ? 64 : B <= 6 ? 42 : B == 7 ? 28 : 20)
-                                      : (B == 3 ? 64 : B == 4 ? 32 : B <= 6 ? 28 : 16);
-  static constexpr int MINB = B == 2 && kSingle ? 4 : B >= 6 && !kSingle ? 2 : 0;
+  static constexpr int LCMAX = B == 1 ? 128
+                               : B <= 3 ? (B == 3 && !kSingle ? 64 : 96)
+                               : B == 4 ? (kSingle ? 64 : 32)
+                               : B <= 6 ? (kSingle ? 42 : 28)
+                                        : 28;
+  static constexpr int LCMIN = B <= 4 || (B == 5 && kSingle) ? LCMAX : B <= 6 ? 16 : 12;
+  static constexpr int MINB = kSingle ? (B == 2 ? 4 : B == 4 ? 3 : 0) : (B >= 6 ? 2 : 0);
   static constexpr int KC = B <= 4 ? 16 : 6;  // pivot blocks D_p^{-1} held at once
-  static constexpr int WVAL = (LC + KC + 1) * B * B;  // values per warp beside the staged row
-  static constexpr int WINT = 2 * LC + 2 * 34;        // ints per warp beside the row's columns
+  static constexpr int WVAL = (KC + 1) * B * B;  // values per warp beside the staged row and the batch
+  static constexpr int WINT = 2 * 34;            // ints per warp beside the row's columns and the batch
 };
+
+int device_sms() {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
+template <int B, typename TV>
+size_t factor_smem_bytes(int chunk, int rc, int lc) {
+  return (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WVAL + (rc + lc) * B * B) * sizeof(TV) +
+         ((size_t)2 * chunk + (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WINT + 2 * lc + rc)) * sizeof(int);
+}
+
+// CTAs that fit into an SM's shared memory (228 KB, 1 KB of it kept per CTA); 0 for
+// more than a CTA may ask for.
+template <int B, typename TV>
+int ctas_by_smem(int chunk, int rc, int lc) {
+  const size_t bytes = factor_smem_bytes<B, TV>(chunk, rc, lc);
+  return bytes > (size_t)kMaxDynamicSmem ? 0 : (int)(228 * 1024 / (bytes + 1024));
+}
 
 // rc: rows of up to rc blocks are staged (at most RC; the widest row of the
 // pattern if that is less).  For b >= 5 none are where the mean row is longer than
 // RC: the buffer would cost a CTA per SM and hold boundary rows only (FP64 b = 8
-// 128x16x8 27-point 28.7 / 25.7 ms).
+// 128x16x8 27-point 28.7 / 25.7 ms).  Nor are any for b >= 7 in FP64 where one CTA
+// fits with the buffer and two without, and one leaves lines waiting: more rows per
+// level than lines resident (b = 8, staged / in place: ILU(2) 96x96x48 78.9 / 58.4 ms,
+// 64x64x32 25.7 / 22.0, ILU(1) 64x64x32 12.3 / 11.1; 280 rows per level, 304 lines
+// resident: 50x45x30 ILU(1) 7.4 / 8.0).
 template <int B, typename TV>
 int staged_rows(const bilu_pattern* p) {
-  constexpr int RC = FactorCap<B, TV>::RC;
-  if (B >= 5 && p->cnt_p > (long long)p->n * RC) return 0;
-  return std::min(RC, p->max_l + 1 + p->max_u);
+  using Cap = FactorCap<B, TV>;
+  if (B >= 5 && p->cnt_p > (long long)p->n * Cap::RC) return 0;
+  const int rc = std::min(Cap::RC, p->max_l + 1 + p->max_u), chunk = p->fact.max_len;
+  const int lines = p->line_len > 0 ? std::max(1, chunk / p->line_len) : 1;
+  if (B >= 7 && !Cap::kSingle && ctas_by_smem<B, TV>(chunk, rc, Cap::LCMIN) < 2 &&
+      ctas_by_smem<B, TV>(chunk, 0, Cap::LCMIN) >= 2 && p->n > (long long)lines * device_sms() * p->nlev_l)
+    return 0;
+  return rc;
 }
 
+// lc: as long as LCMAX where that leaves as many CTAs per SM as LCMIN does
+// (96x96x48 b = 6 FP64 ILU(2), one CTA with 28 entries 48.5 ms, two with fewer 32.2;
+// b = 8 ILU(0) 22.2 / 16.7).
 template <int B, typename TV>
-size_t factor_smem_bytes(int chunk, int rc) {
-  return (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WVAL + rc * B * B) * sizeof(TV) +
-         ((size_t)2 * chunk + (size_t)FactorCap<B, TV>::W * (FactorCap<B, TV>::WINT + rc)) * sizeof(int);
+int batch_entries(int chunk, int rc) {
+  using Cap = FactorCap<B, TV>;
+  const int want = std::min(ctas_by_smem<B, TV>(chunk, rc, Cap::LCMIN), Cap::kSingle ? 3 : 2);
+  int lc = Cap::LCMIN;
+  while (lc < Cap::LCMAX && ctas_by_smem<B, TV>(chunk, rc, lc + 1) >= want) ++lc;
+  return lc;
 }
 
 // Whether a value is finite, and the order of magnitudes, on the integer pipes
@@ -107,7 +146,7 @@ __device__ __forceinline__ bool finite_bits(double v) { return magnitude(v) < 0x
 __device__ __forceinline__ bool finite_bits(float v) { return magnitude(v) < 0x7f800000u; }
 
 // D^{-1} by Gauss-Jordan with partial pivoting on [D | I]: lane c < 2B holds
-// column c in registers (the upper lanes hold nothing and mirror column 0).
+// column c in registers (the lanes above hold zeros).
 // False if a pivot or the result is zero or not finite.
 template <int B, typename TV>
 __device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
@@ -153,8 +192,9 @@ __device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
 }
 
 // Measured before / after (backfill to U' = D^{-1} U, same chunks): 96x96x48
-// ILU(1) b = 3 FP64 6.20 / 5.56 ms, 61x47x33 ILU(2) b = 4 FP32 5.64 / 4.23 ms;
-// per row 37 k cycles, of which 10 k the inverse, 9 k the pivots, 5 k staging.
+// ILU(1) b = 3 FP64 6.20 / 5.56 ms, 61x47x33 ILU(2) b = 4 FP32 5.64 / 4.23 ms (with
+// chunks of one line 2.03); per row 37 k cycles, of which 10 k the inverse, 9 k the
+// pivots, 5 k staging.
 // What bounds it: the FP64 pipe (19 cycles per warp instruction and SM whatever
 // the active lanes) and the chain of dependent rows.  So a row's work is cut to
 // the matching entries of its pivots' U rows, packed over the lanes, with
@@ -163,7 +203,7 @@ __device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
 // only what depends on the last pivots left once those arrive.
 template <int B, typename TV>
 __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MINB) factor_kernel(
-    int32_t n, int32_t chunk, int32_t rc, int32_t nchunks, const int32_t* __restrict__ bnd,
+    int32_t n, int32_t chunk, int32_t rc, int32_t lc_arg, int32_t nchunks, const int32_t* __restrict__ bnd,
     const int32_t* __restrict__ ord, const int32_t* __restrict__ tick,
     const int32_t* __restrict__ lrp, const int32_t* __restrict__ lci,
     const int32_t* __restrict__ urp, const int32_t* __restrict__ uci, TV* f, long long nnz_l,
@@ -171,21 +211,22 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
   using Cap = FactorCap<B, TV>;
   constexpr int BB = B * B;
   constexpr int H = (BB + 31) / 32;
-  constexpr int LC = Cap::LC, KC = Cap::KC;
+  constexpr int KC = Cap::KC;
+  const int lc = Cap::LCMIN == Cap::LCMAX ? Cap::LCMAX : lc_arg;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wvals = Cap::WVAL + rc * BB;
+  const int wvals = Cap::WVAL + (rc + lc) * BB;
   TV* rowv = reinterpret_cast<TV*>(smem_raw) + (size_t)warp * wvals;  // the row being factored
   TV* ub = rowv + rc * BB;  // U_pj of the batch's matches
-  TV* db = ub + LC * BB;    // D_p^{-1}
+  TV* db = ub + lc * BB;    // D_p^{-1}
   TV* aip = db + KC * BB;   // scaled A_ip
   int* fl = reinterpret_cast<int*>(reinterpret_cast<TV*>(smem_raw) + (size_t)Cap::W * wvals);  // ready flags (value =
                                                                                                // chunk id)
   int* s_i = fl + chunk;  // rows of the chunk in local-level order
-  int* cols = s_i + chunk + warp * (Cap::WINT + rc);  // column of each staged slot
+  int* cols = s_i + chunk + warp * (Cap::WINT + 2 * lc + rc);  // column of each staged slot
   int* msrc = cols + rc;    // the batch's matches: U entry,
-  int* mdst = msrc + LC;    // slot in the row
-  int* moff = mdst + LC;    // first match of each pivot of the batch (33)
+  int* mdst = msrc + lc;    // slot in the row
+  int* moff = mdst + lc;    // first match of each pivot of the batch (33)
   int* coff = moff + 34;    // first candidate of each pivot of the batch (33)
   __shared__ int s_c;
   TV* L = f;
@@ -244,8 +285,8 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
       __syncwarp();
       int k0 = 0, s0 = 0;  // the next batch starts with entry s0 of pivot k0's U row
       while (k0 < nl && !dead) {
-        // ---- the batch: whole pivots while their U rows hold at most LC
-        // entries (lane x: pivot k0 + x); of a longer one, LC entries of it
+        // ---- the batch: whole pivots while their U rows hold at most lc
+        // entries (lane x: pivot k0 + x); of a longer one, lc entries of it
         const int np = min(32, nl - k0);
         int p = -1, pb = 0, plen = 0;
         if (lane < np) {
@@ -259,13 +300,13 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
           const int v = __shfl_up_sync(kFull, upto, d);
           if (lane >= d) upto += v;
         }
-        const unsigned fits = __ballot_sync(kFull, lane < np && upto <= LC);
+        const unsigned fits = __ballot_sync(kFull, lane < np && upto <= lc);
         int nfit = __popc(fits), next_s0 = 0;
         const bool slice = nfit == 0;
         if (slice) {
           nfit = 1;
-          next_s0 = s0 + LC;
-          if (lane == 0) upto = plen = LC;
+          next_s0 = s0 + lc;
+          if (lane == 0) upto = plen = lc;
         }
         const int cands = __shfl_sync(kFull, upto, nfit - 1);
         __syncwarp();
@@ -307,22 +348,27 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
             const int at = nm + __popc(m & ((1u << lane) - 1u));
             msrc[at] = src;
             mdst[at] = dst;
-            atomicAdd(&moff[x + 1], 1);
+            if (cands > 32) atomicAdd(&moff[x + 1], 1);
           }
           nm += __popc(m);
+          if (cands <= 32 && lane < nfit)  // all in one go: the matches before each pivot's end
+            moff[lane + 1] = __popc(m & (upto >= 32 ? ~0u : (1u << upto) - 1u));
         }
         __syncwarp();
-        int upm = lane < nfit ? moff[lane + 1] : 0;
+        if (cands > 32) {
+          int upm = lane < nfit ? moff[lane + 1] : 0;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const int v = __shfl_up_sync(kFull, upm, d);
-          if (lane >= d) upm += v;
+          for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(kFull, upm, d);
+            if (lane >= d) upm += v;
+          }
+          __syncwarp();
+          if (lane < nfit) moff[lane + 1] = upm;
+          __syncwarp();
         }
-        __syncwarp();
-        if (lane < nfit) moff[lane + 1] = upm;
-        __syncwarp();
-        // the warp's next row: into L2 while this one waits
-        if (k0 == 0 && s0 == 0) {
+        // the warp's next row: into L2 while this one waits (b = 1: its few bytes are
+        // in lines its neighbours fetch; 96x96x48 ILU(1) FP32 1.87 / 1.74 ms without)
+        if (B > 1 && k0 == 0 && s0 == 0) {
           auto pull = [&](const void* first, size_t bytes) {
             for (size_t o = (size_t)lane * 128; o < bytes; o += 32 * 128)
               asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)first + o));
@@ -354,9 +400,7 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
           run = min(min(run, nfit - x), KC);
           // their D_p^{-1} and matching U_pj, all loads in flight together
           const int m0 = moff[x], mv = (moff[x + run] - m0) * BB, dv = run * BB;
-          // (eight a lane for large blocks, whose batches take many rounds)
-          constexpr int NMAX = B >= 6 ? 8 : 5;
-          constexpr int NB = (KC * BB + 31) / 32 < NMAX ? (KC * BB + 31) / 32 : NMAX;
+          constexpr int NB = (KC * BB + 31) / 32 < 5 ? (KC * BB + 31) / 32 : 5;
           for (int e0 = 0; e0 < dv || e0 < mv; e0 += 32 * NB) {
             TV tu[NB], td[NB];
 #pragma unroll
@@ -418,7 +462,7 @@ __global__ void __launch_bounds__(FactorCap<B, TV>::W * 32, FactorCap<B, TV>::MI
               for (int m = 0; m < B; ++m) s = fma(aip[m * B + r], upj[m], s);
               return s;
             };
-            if (B >= 6 && !staged) {
+            if (B >= 7 && !staged) {
               // in place: two elements a lane at a time, both read before either is
               // written (a pivot's matches are different blocks); one at a time is a
               // chain of round trips (b = 7 FP32 160x20x20 27-point 34.4 / 27.6 ms)
@@ -523,13 +567,6 @@ __global__ void __launch_bounds__(256) scale_upper_kernel(int32_t n, const int32
   }
 }
 
-int device_sms() {
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms > 0 ? sms : 1;
-}
-
 template <typename TV>
 int launch_backfill_t(const bilu_pattern* p, int32_t b, const double* a_vals, TV* f, void* stream) {
   const long long total = p->nslots() * (long long)b * b;
@@ -557,7 +594,8 @@ int launch_factor_t(const bilu_pattern* p, int32_t b, TV* f, int32_t* header, in
   const long long spin = trisolve_config().spin_ns;
   BILU_DISPATCH_B(b, {
     const int rc = staged_rows<B, TV>(p);
-    const size_t smem = factor_smem_bytes<B, TV>(chunk, rc);
+    const int lc = batch_entries<B, TV>(chunk, rc);
+    const size_t smem = factor_smem_bytes<B, TV>(chunk, rc, lc);
     static LaunchCache cache;
     const int per_sm = cache.ctas_per_sm(current_device(), smem, [](size_t bytes) {
       cudaFuncSetAttribute(factor_kernel<B, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
@@ -567,7 +605,7 @@ int launch_factor_t(const bilu_pattern* p, int32_t b, TV* f, int32_t* header, in
     });
     const int grid = std::max(1, std::min(nchunks, per_sm * sms));
     ProfScope ps(BILU_PROF_FACTOR, stream);
-    factor_kernel<B, TV><<<grid, FactorCap<B, TV>::W * 32, smem, s>>>(n, chunk, rc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
+    factor_kernel<B, TV><<<grid, FactorCap<B, TV>::W * 32, smem, s>>>(n, chunk, rc, lc, nchunks, p->fact.d_bnd, p->fact.d_ord_l, p->fact.d_tick_l, p->d_lrp, p->d_lci,
                                                             p->d_urp, p->d_uci, f, p->nnz_l(), header, done,
                                                             spin);
   });

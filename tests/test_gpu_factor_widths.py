@@ -37,6 +37,23 @@ def _blocks(widths, b, seed):
     (7, (17, 18, 24)), (7, (25, 29, 30)), (7, (50, 3)), (8, (17, 18)), (8, (20, 21, 22)), (8, (24,)), (8, (25, 40)),
 ])
 def test_batch_and_buffer_edges(libbilu, b, widths):
+    _check(b, widths)
+
+
+@pytest.mark.parametrize("rows", [17, 512, 1024])
+@pytest.mark.parametrize("b", [1, 3, 5, 6, 7, 8])
+def test_chunk_lengths(libbilu, b, rows):
+    """The batch and the buffer shrink with the rows per chunk that shared memory also holds (1024: 8 KB)."""
+    import paper_1703_01325_gb300.bilu as B
+    old = B.bilu_get_factor_chunk()
+    try:
+        B.bilu_set_factor_chunk(rows)
+        _check(b, (23, 22) * (30 if b < 5 else 24))
+    finally:
+        B.bilu_set_factor_chunk(old)
+
+
+def _check(b, widths):
     import paper_1703_01325_gb300.bilu as B
     torch.cuda.set_device(0)
     S = _blocks(widths, b, seed=13 * b + sum(widths))
