@@ -110,8 +110,12 @@ int bilu_pattern_export(const bilu_pattern* p, int32_t* row_ptr, int32_t* col_id
 /*
  * bilu_pattern_upload -- copy the pattern's integer structure to the current
  * device and build the schedules of the sync-free factorization and solves
- * (set-up; allocates device memory owned by the handle, about
- * 4*(4n + nnz_l + nnz_u + nnz_a) bytes).  Synchronises the stream.  Needed
+ * (set-up; allocates device memory owned by the handle: about
+ * 4*(3n + 2 nnz_l + 2 nnz_u) bytes for the structure and the backfill map, 8n for
+ * the solves' schedule, as much again where a second one is built, 4n for the
+ * factorization's; while it runs up to 33 bytes a row, or about 20 per block of
+ * the larger triangle, of scratch).  Synchronises the stream.  Without memory for the second
+ * schedule the call goes on without it.  Needed
  * before bilu_factor, bilu_apply and the solvers, which return
  * BILU_ERR_STATE without it.
  */
@@ -429,11 +433,14 @@ int gmres_solve(const bilu_pattern* p, const bilu_bsr* A, const double* d_factor
 
 /*
  * bilu_symbolic_gpu -- the same P', fill levels and Eq. 4 levels as
- * bilu_symbolic (bit for bit), computed on the current device: Algorithm 3's
- * row merges with one warp per row (rows in ascending order, row i waiting,
- * bounded, for each pivot row p < i it merges), then the completion of the
- * pattern -- row pointers (device scans), the L / U' split, the Eq. 4 levels
- * (a sync-free longest-path pass per triangle, one warp per row) and the
+ * bilu_symbolic (bit for bit), computed on the current device.  For k <= 3 each
+ * row of P' is found from A alone, by the paths that make its fill (one warp per
+ * row, no row waits for another).  For larger k, or where a row meets more than
+ * 384 columns on the way, by Algorithm 3's row merges: one warp per row, rows in
+ * ascending order, row i waiting, bounded, for each pivot row p < i it merges.
+ * Then the completion of the pattern -- row pointers (device scans), the L / U'
+ * split, the Eq. 4 levels (a sync-free longest-path pass per triangle, one warp
+ * per row, or per 32 rows where every grid line is whole runs of 32) and the
  * backfill map of Algorithm 5 -- also on the device, straight into the
  * handle's device copy.  Inputs are host arrays as for bilu_symbolic.  The
  * returned handle lives on this device; bilu_pattern_upload on the same
@@ -442,8 +449,10 @@ int gmres_solve(const bilu_pattern* p, const bilu_bsr* A, const double* d_factor
  * bilu_pattern_transpose, bilu_schedule_export, an upload to another device).
  *   row_capacity in [1, 8192]: the most entries any row of P' may hold; a row
  *   that outgrows it returns BILU_ERR_OOM (retry with a larger capacity).
- *   Device scratch of about 8 * n * row_capacity bytes is allocated and freed
- *   inside the call; the stream is synchronised.  BILU_ERR_TIMEOUT if a wait
+ *   Device scratch of about 4 * (11 n + nnz_a) bytes is allocated and freed
+ *   inside the call, for the merges 8 * n * row_capacity bytes more (BILU_ERR_OOM
+ *   if they cannot be had, so with a large row_capacity that can depend on one
+ *   row); the stream is synchronised.  BILU_ERR_TIMEOUT if a wait
  *   exceeds the spin limit (bilu_set_spin_limit_ns).
  */
 int bilu_symbolic_gpu(int32_t n, const int32_t* row_ptr, const int32_t* col_idx, int32_t k, int32_t row_capacity,

@@ -178,8 +178,8 @@ def bilu_symbolic(n: int, row_ptr, col_idx, k: int) -> Pattern:
 
 
 def bilu_symbolic_gpu(n: int, row_ptr, col_idx, k: int, row_capacity: int = 256, stream=None) -> Pattern:
-    """The same pattern as bilu_symbolic, with Algorithm 3's row merges run on
-    the current CUDA device (bilu_symbolic_gpu)."""
+    """The same pattern as bilu_symbolic, computed on the current CUDA device
+    (bilu_symbolic_gpu)."""
     rp = _host_i32(row_ptr)
     ci = _host_i32(col_idx)
     if len(rp) != n + 1:

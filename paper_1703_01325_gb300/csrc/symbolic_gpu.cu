@@ -206,7 +206,11 @@ __global__ void __launch_bounds__(kSymWarps * 32) symbolic_kernel(
 // Statistics words (device scratch).
 enum StatWord : int { kMaxL = 0, kMaxU = 1, kNlevL = 2, kNlevU = 3, kBadPattern = 4, kLongest = 5, kStatWords = 8 };
 
-constexpr int kMaxPathLevel = 3;  // longer walks revisit more than a merge does
+// The largest k that goes by paths: what it was built and tested for, not a measured
+// crossing (whole call, paths / merges, ms: 64x64x32 7-point k = 4 12.8 / 54.3, k = 6
+// 39.4 / 102.6; 27-point 40x40x20 k = 3 7.2 / 12.7, k = 4, whose rows do not fit the
+// table, 27.4 / 26.6).
+constexpr int kMaxPathLevel = 3;
 constexpr int kPathWarps = 4;
 constexpr int kNever = INT_MAX;
 
