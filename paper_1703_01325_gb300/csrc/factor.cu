@@ -193,7 +193,7 @@ __device__ __forceinline__ bool invert_columns(TV (&col)[B], int lane) {
 
 // Measured before / after (backfill to U' = D^{-1} U, same chunks): 96x96x48
 // ILU(1) b = 3 FP64 6.20 / 5.56 ms, 61x47x33 ILU(2) b = 4 FP32 5.64 / 4.23 ms (with
-// chunks of one line 2.03); per row 37 k cycles, of which 10 k the inverse, 9 k the
+// chunks of one line 2.10); per row 37 k cycles, of which 10 k the inverse, 9 k the
 // pivots, 5 k staging.
 // What bounds it: the FP64 pipe (19 cycles per warp instruction and SM whatever
 // the active lanes) and the chain of dependent rows.  So a row's work is cut to
